@@ -37,6 +37,7 @@ UNITS = {
     "loss.cu": [],
     "static_scratch.cu": [],
     "query.cu": [],
+    "query_wide.cu": [],
     "color.cu": [],
 }
 

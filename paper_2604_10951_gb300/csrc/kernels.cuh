@@ -158,10 +158,14 @@ cudaError_t launch_render_backward(const Cams& cams, const RParams& P, const Bwd
 // query-guided instance labels (query.cu): l_ins [N, nq] (F32 or BF16) from
 // BF16 f_ins [N, dim] and f_q [nq, dim]; nq in {16, 32, ..., 256}, dim in
 // {16, 32, ..., 128}; *err set to 1 if a bounded wait on the tensor cores expired
-size_t query_labels_smem(int nq, int dim);
 cudaError_t launch_query_labels(int64_t N, int nq, int dim, const void* f_ins, const float* means, const void* f_q,
                                 const float* p_q, const float* prec, void* out, int out_bf16, int32_t* err,
                                 int num_sms, cudaStream_t stream);
+
+// ... for many queries (query_wide.cu)
+cudaError_t launch_query_wide(int64_t N, int nq, int dim, const void* f_ins, const float* means, const void* f_q,
+                              const float* p_q, const float* prec, void* out, int out_bf16, int32_t* err, int num_sms,
+                              cudaStream_t stream);
 
 // view-dependent colours (color.cu): item directions at binning, item colours
 // before the forward render

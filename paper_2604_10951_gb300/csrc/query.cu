@@ -1,4 +1,5 @@
-// Query-guided instance labels (Sec. 3.3) on the 5th-generation tensor cores.
+// Query-guided instance labels (Sec. 3.3) on the 5th-generation tensor cores:
+// the entry, and the kernel for few queries (query_wide.cu has the one for many).
 //
 // For every scene Gaussian g and instance query q:
 //   S = sigmoid(f_q . f_ins(g)),  D = exp(-1/2 d^T Sigma_q^-1 d), d = p_g - p_q,
@@ -21,11 +22,7 @@
 // Every wait on the MMA's mbarrier is bounded: on expiry the kernel raises
 // the caller's error word, stops taking tiles, frees its tensor memory and
 // returns.
-#include "fss_internal.cuh"
-#include "kernels.cuh"
-#include "render_common.cuh"
-
-#include <cuda_bf16.h>
+#include "query_common.cuh"
 
 #include <algorithm>
 
@@ -33,42 +30,7 @@ namespace fss {
 
 namespace {
 
-constexpr int QM = 128;        // Gaussians per tile (MMA M)
 constexpr int QTHREADS = 128;  // warp w reads TMEM lanes 32 w .. 32 w + 31
-constexpr int QWAIT = 1 << 22; // try_wait rounds before giving up
-constexpr float QLOG2E = 1.4426950408889634f;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// shared-memory matrix descriptor: start, leading (K) and stride (row-group)
-// byte offsets, descriptor version 1, no swizzle
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
-           (1ull << 46);
-}
-
-// instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
-// K-major, N = n, M = 128
-__host__ __device__ constexpr uint32_t mma_idesc(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(QM >> 4) << 24);
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (int i = 0; i < QWAIT; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     uint32_t r[16];
@@ -291,6 +253,8 @@ __global__ void __launch_bounds__(QTHREADS, KC <= 4 ? 8 : 1) k_query_labels(int6
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
+size_t query_labels_smem(int nq, int dim) { return (size_t)QM * dim * 2 + (size_t)nq * dim * 2 + (size_t)nq * 48; }
+
 template <int KC>
 cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, const void* f_q, const float* p_q,
                       const float* prec, void* out, int out_bf16, int32_t* err, int num_sms, cudaStream_t stream) {
@@ -326,14 +290,29 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
     return e;
 }
 
-}  // namespace
+// Which kernel, from both timed over 2,000 to 1.3M Gaussians, 16 to 192
+// queries and 16 to 128 channels.  The kernel above reads a query's parameters
+// once per thread and label (query_wide.cu: once per two Gaussians) and stores
+// its rows uncoalesced, but keeps eight small CTAs per SM, so it is ahead where
+// a tile is little work: 500k x 32 x 32 takes 27.1 us with BF16 labels and 38.2
+// with FP32 against 31.1 and 36.7; 80 x 48 59.2 and 81.2 against 61.1 and 67.7.
+// FP32 labels store twice the bytes: from 80 queries on query_wide.cu is ahead
+// (112 x 64: 123 / 91 us).  BF16 labels gain less (112 x 64 91.2 / 84.5, 128 x
+// 96 120.5 / 99.2) and lose below 100k Gaussians (50,000 x 112 x 48 14.1 / 16.2)
+// and above 96 channels, where shared memory leaves query_wide.cu fewer
+// Gaussians per SM (128 x 128 with 1.3M: 292 / 332).
+bool wide_queries(int64_t N, int nq, int dim, bool bf16) {
+    return bf16 ? nq >= 96 && dim <= 96 && N >= 100000 : nq >= 80;
+}
 
-size_t query_labels_smem(int nq, int dim) { return (size_t)QM * dim * 2 + (size_t)nq * dim * 2 + (size_t)nq * 48; }
+}  // namespace
 
 cudaError_t launch_query_labels(int64_t N, int nq, int dim, const void* f_ins, const float* means, const void* f_q,
                                 const float* p_q, const float* prec, void* out, int out_bf16, int32_t* err,
                                 int num_sms, cudaStream_t stream) {
     if (N <= 0) return cudaSuccess;
+    if (wide_queries(N, nq, dim, out_bf16 != 0))
+        return launch_query_wide(N, nq, dim, f_ins, means, f_q, p_q, prec, out, out_bf16, err, num_sms, stream);
     switch (dim) {
         case 16: return launch_kc<2>(N, nq, f_ins, means, f_q, p_q, prec, out, out_bf16, err, num_sms, stream);
         case 32: return launch_kc<4>(N, nq, f_ins, means, f_q, p_q, prec, out, out_bf16, err, num_sms, stream);
