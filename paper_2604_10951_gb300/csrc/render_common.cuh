@@ -183,6 +183,57 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// ... all but this thread's most recent group
+__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// One warp's walk over its tile's list, without barriers between the warps: 32
+// list positions at a time, the records whose mask has the warp's bit copied
+// asynchronously into the warp's own half of a double buffer (a lane's record
+// in the lane's place) while the warp works on the other half.
+// ---------------------------------------------------------------------------
+struct WarpStage {
+    float4 r0[32], r1[32], r2[32], oc[32];  // adjugate rows; (o, r, g, b)
+};
+
+// list item and warp mask of position j (mask 0 outside [0, n))
+struct ListEntry {
+    uint32_t item, mask;
+};
+__device__ __forceinline__ ListEntry list_entry(const uint32_t* list, const uint32_t* masks, int j, int n) {
+    ListEntry e{0u, 0u};
+    if (j >= 0 && j < n) {
+        e.item = list[j];
+        e.mask = masks[j];
+    }
+    return e;
+}
+
+// Starts the copies of a chunk's records that the warp meets (one commit
+// group per call) and returns them as a lane mask.
+__device__ __forceinline__ uint32_t stage_chunk(WarpStage& s, const ListEntry& e, uint32_t wbit, const float4* rec,
+                                                const float* rgbv, int64_t vbase, int64_t N, Status* st) {
+    const int lane = threadIdx.x & 31;
+    const int64_t sp = (int64_t)e.item - vbase;
+    const bool hit = (e.mask & wbit) && in_bounds(st, SITE_ITEM, sp, N);  // check build: a bad item is skipped
+    if (hit) {
+        const float4* r = rec + 4 * (size_t)e.item;
+        cp_async16(&s.r0[lane], r, 16);
+        cp_async16(&s.r1[lane], r + 1, 16);
+        cp_async16(&s.r2[lane], r + 2, 16);
+        cp_async4(&s.oc[lane].x, r + 3);
+        cp_async4(&s.oc[lane].y, rgbv + 3 * sp);
+        cp_async4(&s.oc[lane].z, rgbv + 3 * sp + 1);
+        cp_async4(&s.oc[lane].w, rgbv + 3 * sp + 2);
+    }
+    cp_async_commit();
+    return __ballot_sync(0xffffffffu, hit);
+}
+
 // Division by a divisor fixed for the whole kernel (d >= 1, 0 <= n < 2^24),
 // without the ~20-instruction integer division: a float reciprocal guess
 // corrected by one step either way.
@@ -448,25 +499,25 @@ __device__ __forceinline__ int argmax_channel(unsigned long long key) {
     return (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
 }
 
-// Launch of a render kernel over the tiles (one CTA per tile, or one resident
-// wave for the persistent schedule), recording the measurement hook after it.
+// Launch of a render kernel over the tiles (`parts` CTAs per tile, or one
+// resident wave for the persistent schedule), recording the measurement hook after it.
 template <typename KernelT>
 inline cudaError_t launch_tiles(KernelT kern, int threads, size_t smem, const Cams& cams, const RParams& P, const FwdArgs& a,
-                               const AuxOut& x, int num_sms, cudaStream_t stream) {
+                               const AuxOut& x, int num_sms, cudaStream_t stream, int parts = 1) {
     cudaError_t e = cudaSuccess;
     if (smem + 2048 > 48 * 1024) {  // above the default limit with the kernels' static shared memory (< 2 KB)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    int grid = cams.total_tiles;
+    int64_t units = (int64_t)cams.total_tiles * parts;
     if (a.persistent) {
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
         if (e != cudaSuccess) return e;
-        grid = std::min(cams.total_tiles, max(1, per_sm) * num_sms);
+        units = std::min<int64_t>(units, (int64_t)std::max(1, per_sm) * num_sms);
     }
-    if (grid <= 0) return cudaSuccess;
-    kern<<<grid, threads, smem, stream>>>(cams, P, a, x);
+    if (units <= 0) return cudaSuccess;
+    kern<<<(unsigned)units, threads, smem, stream>>>(cams, P, a, x);
     e = cudaGetLastError();
     if (e == cudaSuccess) kernel_mark(stream);
     return e;

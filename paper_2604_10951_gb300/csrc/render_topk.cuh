@@ -29,6 +29,7 @@
 #include "fss_internal.cuh"
 #include "kernels.cuh"
 #include "render_common.cuh"
+#include "render_topk_wide.cuh"
 #include "sort.cuh"
 
 #include <algorithm>
@@ -437,23 +438,15 @@ cudaError_t launch_topk(const Cams& cams, const RParams& P, const FwdArgs& a, co
                             std::max(smem(8), SORT_SMEM_BYTES), cams, P, a, x, num_sms, s);
     if (x.loss.loss)
         return launch_tiles(k_render_topk<TS, 8, FT, false, false, true>, NT, smem(8), cams, P, a, x, num_sms, s);
-    // variants (first-K selection, sensor outputs) need unsorted or few slots: two capacities
-    if (P.select == FSS_SELECT_FRONT) {
-        if (aux) {
-            if (P.K <= 8) return launch_tiles(k_render_topk<TS, 8, FT, true, true>, NT, smem(8), cams, P, a, x, num_sms, s);
-            return launch_tiles(k_render_topk<TS, 32, FT, true, true>, NT, smem(32), cams, P, a, x, num_sms, s);
-        }
-        if (P.K <= 8) return launch_tiles(k_render_topk<TS, 8, FT, true, false>, NT, smem(8), cams, P, a, x, num_sms, s);
-        return launch_tiles(k_render_topk<TS, 32, FT, true, false>, NT, smem(32), cams, P, a, x, num_sms, s);
-    }
-    if (aux) {
-        if (P.K <= 8) return launch_tiles(k_render_topk<TS, 8, FT, false, true>, NT, smem(8), cams, P, a, x, num_sms, s);
-        return launch_tiles(k_render_topk<TS, 32, FT, false, true>, NT, smem(32), cams, P, a, x, num_sms, s);
-    }
+    // sets of more than eight entries live in shared memory (render_topk_wide.cuh):
+    // in registers K = 9..16 take 112 registers and K = 32 220
+    if (P.K > 8) return launch_topk_wide<TS, FT>(cams, P, a, x, num_sms, s);
+    if (P.select == FSS_SELECT_FRONT)
+        return aux ? launch_tiles(k_render_topk<TS, 8, FT, true, true>, NT, smem(8), cams, P, a, x, num_sms, s)
+                   : launch_tiles(k_render_topk<TS, 8, FT, true, false>, NT, smem(8), cams, P, a, x, num_sms, s);
+    if (aux) return launch_tiles(k_render_topk<TS, 8, FT, false, true>, NT, smem(8), cams, P, a, x, num_sms, s);
     if (P.K <= 4) return launch_tiles(k_render_topk<TS, 4, FT, false, false>, NT, smem(4), cams, P, a, x, num_sms, s);
-    if (P.K <= 8) return launch_tiles(k_render_topk<TS, 8, FT, false, false>, NT, smem(8), cams, P, a, x, num_sms, s);
-    if (P.K <= 16) return launch_tiles(k_render_topk<TS, 16, FT, false, false>, NT, smem(16), cams, P, a, x, num_sms, s);
-    return launch_tiles(k_render_topk<TS, 32, FT, false, false>, NT, smem(32), cams, P, a, x, num_sms, s);
+    return launch_tiles(k_render_topk<TS, 8, FT, false, false>, NT, smem(8), cams, P, a, x, num_sms, s);
 }
 
 template <typename FT>
