@@ -10,7 +10,6 @@
 
 namespace fss {
 
-constexpr int BATCH = 256;   // staged records per batch (Top-K kernels)
 constexpr int FBATCH = 64;   // staged records + feature rows per batch (full kernels)
 constexpr float NEG_HALF_LOG2E = -0.72134752044448170f;  // exp(-r/2) = 2^(r * this)
 
