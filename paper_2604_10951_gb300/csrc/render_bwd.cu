@@ -13,12 +13,13 @@
 //             grouped by surfel in shared memory first, so each surfel's
 //             feature row is read once and costs one row of 16-byte vector
 //             reductions per tile.
-// k_bwd_geo   one CTA per tile, one thread per pixel: back-to-front replay;
-//             per staged surfel the warp reduce-scatters its 13 partial
-//             derivatives (adjugate rows 9, opacity 1, colour 3) and the
-//             CTA flushes one row of vector reductions per surfel and tile.
-//             The full-accumulation variant also forms c_j . dL/dF inline
-//             and reduce-scatters the feature gradient.
+// k_bwd_geo_topk one warp per 8 x 4 pixel block: back-to-front replay; per
+//             surfel the warp reduce-scatters its 13 partial derivatives
+//             (adjugate rows 9, opacity 1, colour 3) and adds them to the
+//             surfel's gradient row.
+// k_bwd_geo_full (K = 0) the same with a CTA per tile: it also forms c_j . dL/dF
+//             inline and reduce-scatters the feature gradient, and flushes one
+//             row of vector reductions per surfel and tile.
 // k_bwd_project one thread per surfel: adjugate-row gradients -> homography
 //             columns -> means, scales, quaternions; sums the views.
 // k_feat_out  writes every row of the feature gradient (zeros for surfels
@@ -35,7 +36,6 @@ namespace fss {
 
 namespace {
 
-constexpr int BB = 128;      // staged surfels per backward batch
 constexpr int BWD_FEAT_THREADS = 256;
 
 // reduce-scatter of V values (power of two, 2..32 per lane...) across a warp:
@@ -68,7 +68,7 @@ __device__ __forceinline__ void reduce_scatter(float* v) {
 
 // ---------------------------------------------------------------------------
 // k_bwd_feat (Top-K): per selected (pixel x, k) with surfel i, the dot
-// c_i . dL/dF(x) (read by k_bwd_geo) and the feature gradient sum over x of
+// c_i . dL/dF(x) (read by k_bwd_geo_topk) and the feature gradient sum over x of
 // w_i(x) dL/dF(x), grouped per tile
 //
 // Per tile (and per chunk of at most ECAP (pixel, k) entries):
@@ -411,13 +411,13 @@ __global__ void __launch_bounds__(BWD_FEAT_THREADS, 4) k_bwd_feat(const __grid_c
 }
 
 // ---------------------------------------------------------------------------
-// k_bwd_geo: back-to-front replay (Top-K and full accumulation)
+// k_bwd_geo_full: back-to-front replay of the full accumulation (K = 0)
 // ---------------------------------------------------------------------------
-template <int TS, bool FULL, int CMAX, typename FT, bool VAR>
-__global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cams cams,
+template <int TS, int CMAX, typename FT, bool VAR>
+__global__ void __launch_bounds__(TS * TS) k_bwd_geo_full(const __grid_constant__ Cams cams,
                                                      const __grid_constant__ RParams P, const BwdArgs a) {
     constexpr int NT = TS * TS;
-    constexpr int NB = FULL ? FBATCH : BB;
+    constexpr int NB = FBATCH;
     extern __shared__ __align__(16) unsigned char smem[];
     float4* s_r0 = reinterpret_cast<float4*>(smem);
     float4* s_r1 = s_r0 + NB;
@@ -425,16 +425,16 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
     float4* s_oc = s_r2 + NB;                                  // (o, r, g, b)
     uint32_t* s_wm = reinterpret_cast<uint32_t*>(s_oc + NB);   // warps the footprint reaches
     float* s_g = reinterpret_cast<float*>(s_wm + 2 * NB);      // [NB][16] partial derivatives
-    float* s_f = s_g + NB * 16;    // FULL: [NB][C] features
-    float* s_gf = s_f + (FULL ? NB * P.C : 0);  // FULL: [NB][C] feature gradients
+    float* s_f = s_g + NB * 16;    // [NB][C] features
+    float* s_gf = s_f + NB * P.C;  // [NB][C] feature gradients
     __shared__ int s_max;
     __shared__ int s_tile;
-    __shared__ uint32_t s_bits[NT / 32][BB / 32];  // per warp: the staged surfels its block meets
+    __shared__ uint32_t s_bits[NT / 32][NB / 32];  // per warp: the staged surfels its block meets
 
     if (a.st->err) return;
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t wbit = 1u << (tid >> 5);
-    const int C = P.C, K = P.K;
+    const int C = P.C;
     for (int t = next_tile_q(a.persistent, &a.st->work_geo, &s_tile, true, cams); t < cams.total_tiles;
          t = next_tile_q(a.persistent, &a.st->work_geo, &s_tile, false, cams)) {
     const int view = view_of_tile(cams, t);
@@ -447,23 +447,17 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
     const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
     const int2 rg = checked_range(a.ranges, t, P.pair_cap, a.st);
     const int64_t vbase = (int64_t)view * P.N;
-    // VAR instances carry the variants (renormalised Top-K, spherical-harmonic
-    // item colours, low-pass filter), read from the parameters; the plain
-    // instance keeps its code as it is
+    // VAR instances carry the variants (spherical-harmonic item colours, low-pass
+    // filter), read from the parameters; the plain instance keeps its code as it is
     const float* __restrict__ rgbv = a.rgb + (VAR && P.color_sh ? 3 * vbase : 0);
     const int64_t pix = cam.pix_off + (int64_t)py * cam.W + px;
     const FT* __restrict__ feats = reinterpret_cast<const FT*>(a.feats);
 
     int nstop = 0;
     float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
-    int kk = -1, next_pos = -1;
-    float next_dot = 0.0f;
-    // a selected surfel adds rn_a * dot + rn_b to what its weight multiplies:
-    // the dot itself, or (dot - F.dL/dF) / W for the renormalised variant
-    float rn_a = 1.0f, rn_b = 0.0f;
-    float dfr[FULL ? CMAX : 1];
+    float dfr[CMAX];
 #pragma unroll
-    for (int c = 0; c < (FULL ? CMAX : 1); ++c) dfr[c] = 0.0f;
+    for (int c = 0; c < CMAX; ++c) dfr[c] = 0.0f;
     if (inside) {
         nstop = a.saved_nstop[pix];
         T = a.out_T[pix];
@@ -471,28 +465,9 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
         gg = a.d_rgb[3 * pix + 1];
         gb = a.d_rgb[3 * pix + 2];
         Sh = P.bg[0] * gr + P.bg[1] * gg + P.bg[2] * gb + (a.d_T ? a.d_T[pix] : 0.0f);
-        if (!FULL) {
-            for (kk = K - 1; kk >= 0; --kk)
-                if (a.saved_pos[pix * K + kk] >= 0) break;
-            if (kk >= 0) {
-                next_pos = a.saved_pos[pix * K + kk];
-                next_dot = a.dots[pix * K + kk];
-            }
-            if (VAR && P.renorm) {  // entries 0..kk are the selected ones, front to back
-                float ws = 0.0f, wd = 0.0f;
-                for (int k2 = 0; k2 <= kk; ++k2) {
-                    const float wv = a.saved_w[pix * K + k2];
-                    ws += wv;
-                    wd = fmaf(wv, a.dots[pix * K + k2], wd);
-                }
-                rn_a = ws > 0.0f ? 1.0f / ws : 0.0f;
-                rn_b = -wd * rn_a * rn_a;
-            }
-        } else {
-            const FT* dF = reinterpret_cast<const FT*>(a.d_feat) + pix * C;
+        const FT* dF = reinterpret_cast<const FT*>(a.d_feat) + pix * C;
 #pragma unroll
-            for (int c = 0; c < (FULL ? CMAX : 1); ++c) dfr[c] = c < C ? FeatVec<FT>::one(dF + c) : 0.0f;
-        }
+        for (int c = 0; c < CMAX; ++c) dfr[c] = c < C ? FeatVec<FT>::one(dF + c) : 0.0f;
     }
     if (tid == 0) s_max = 0;
     __syncthreads();
@@ -520,7 +495,7 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
             s_wm[j] = a.masks[rg.x + b_start + j];
         }
         for (int i = tid; i < cnt * 16; i += NT) s_g[i] = 0.0f;
-        if (FULL) {
+        {
             constexpr int E = FeatVec<FT>::E;
             const int nvec = C / E, rpi = NT / nvec, r0 = tid / nvec, vv = tid - r0 * nvec;
             for (int j = r0; r0 < rpi && j < cnt; j += rpi) {
@@ -563,28 +538,19 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
                 const float Tj = T * rcp_approx(1.0f - alpha);
                 w = alpha * Tj;
                 float s = oc.y * gr + oc.z * gg + oc.w * gb;
-                if (!FULL) {
-                    if (pos == next_pos) {
-                        s += VAR ? fmaf(next_dot, rn_a, rn_b) : next_dot;
-                        --kk;
-                        next_pos = kk >= 0 ? a.saved_pos[pix * K + kk] : -1;
-                        next_dot = kk >= 0 ? a.dots[pix * K + kk] : 0.0f;
-                    }
-                } else {
-                    const float4* fr = reinterpret_cast<const float4*>(s_f + j * C);
-                    float d0 = 0.0f, d1 = 0.0f;
+                const float4* fr = reinterpret_cast<const float4*>(s_f + j * C);
+                float d0 = 0.0f, d1 = 0.0f;
 #pragma unroll
-                    for (int c4 = 0; c4 < CMAX / 4; ++c4) {
-                        if (4 * c4 < C) {
-                            const float4 fv = fr[c4];
-                            d0 = fmaf(fv.x, dfr[4 * c4], d0);
-                            d1 = fmaf(fv.y, dfr[4 * c4 + 1], d1);
-                            d0 = fmaf(fv.z, dfr[4 * c4 + 2], d0);
-                            d1 = fmaf(fv.w, dfr[4 * c4 + 3], d1);
-                        }
+                for (int c4 = 0; c4 < CMAX / 4; ++c4) {
+                    if (4 * c4 < C) {
+                        const float4 fv = fr[c4];
+                        d0 = fmaf(fv.x, dfr[4 * c4], d0);
+                        d1 = fmaf(fv.y, dfr[4 * c4 + 1], d1);
+                        d0 = fmaf(fv.z, dfr[4 * c4 + 2], d0);
+                        d1 = fmaf(fv.w, dfr[4 * c4 + 3], d1);
                     }
-                    s += d0 + d1;
                 }
+                s += d0 + d1;
                 const float dal = Tj * (s - Sh);
                 Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
                 g[10] = w * gr;
@@ -609,7 +575,7 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
             if (__any_sync(0xffffffffu, contrib)) {
                 reduce_scatter<16>(g);  // lane l holds value l >> 1
                 if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13)) atomicAdd(&s_g[j * 16 + (lane >> 1)], g[0]);
-                if (FULL) {
+                {
 #pragma unroll
                     for (int c0 = 0; c0 < CMAX; c0 += 32) {
                         if (c0 < C) {
@@ -645,7 +611,7 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
             else
                 atomicAdd(dst + 12, v[12]);
         }
-        if (FULL) {
+        {
             const int c4 = C / 4;
             for (int idx = tid; idx < cnt * c4; idx += NT) {
                 const int j = idx / c4, q = idx - j * c4;
@@ -661,6 +627,204 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo(const __grid_constant__ Cam
     }
     __syncthreads();
     }  // tiles
+}
+
+// ---------------------------------------------------------------------------
+// k_bwd_geo_topk: back-to-front replay of the Top-K render, one warp per 8 x 4
+// pixel block, each warp on its own
+// ---------------------------------------------------------------------------
+// The warp walks its tile's list backwards 32 positions at a time (stage_chunk,
+// with the surfels' gradient slots beside the records); per surfel its lanes'
+// 13 partial derivatives are reduce-scattered over the warp, and 13 lanes add
+// the sums to the surfel's gradient row in L2 (64 consecutive bytes, one
+// request).  Partial sums used to be gathered per tile in shared memory, behind
+// the barriers of the staging (1.8 cycles per issued instruction there): 98 us for a
+// 640 x 480 frame of 500k surfels, 88 here; 1296 x 968 with K = 24 324 / 305.
+// Bound by instruction issue: about 40 of a warp evaluation's instructions are
+// the record, the ray and the derivatives, 55 the reduce-scatter.
+constexpr int GEO_THREADS = 128;  // threads per CTA (64 for 8 x 8 tiles): parts of a tile
+
+struct GeoStage {
+    WarpStage st[2];
+    int32_t slot[2][32];
+};
+
+// warp sums of v[0..12]: afterwards an even lane l < 26 holds the sum of v[l >> 1]
+__device__ __forceinline__ void reduce_scatter13(float (&v)[13]) {
+    const int lane = threadIdx.x & 31;
+    const bool up = (lane & 16) != 0;
+    // values i and 8 + i in pairs for i < 5, values 5..7 summed by both halves
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const float send = up ? v[i] : v[i + 8];
+        const float keep = up ? v[i + 8] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+#pragma unroll
+    for (int i = 5; i < 8; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
+#pragma unroll
+    for (int o = 8, n = 8; o > 1; o >>= 1, n >>= 1) {
+        const bool u = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const float send = u ? v[i] : v[i + n / 2];
+            const float keep = u ? v[i + n / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+template <int TS, bool VAR>
+__global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
+                                  1024 / (TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS))
+    k_bwd_geo_topk(const __grid_constant__ Cams cams, const __grid_constant__ RParams P, const BwdArgs a) {
+    constexpr int NT = TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS, NW = NT / 32, PARTS = TS * TS / NT;
+    constexpr unsigned ALL = 0xffffffffu;
+    __shared__ __align__(16) GeoStage s_stage[NW];
+    __shared__ int s_work;
+    if (a.st->err) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    GeoStage& G = s_stage[warp];
+    const int K = P.K, total = cams.total_tiles * PARTS;
+    for (bool first = true;; first = false) {
+        int u;  // this CTA's next part of a tile (heavy tiles first)
+        if (!a.persistent) {
+            u = first ? (int)blockIdx.x : INT_MAX;
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) s_work = (int)atomicAdd(&a.st->work_geo, 1u);
+            __syncthreads();
+            u = s_work;
+        }
+        if (u >= total) return;
+        const int t = cams.tile_order ? cams.tile_order[u / PARTS] : u / PARTS;
+        const int wb = (u % PARTS) * NW + warp;  // this warp's block of the tile
+        const uint32_t wbit = 1u << wb;
+        const int view = view_of_tile(cams, t);
+        const CamDev& cam = cams.c[view];
+        const int lt = t - cam.tile_off;
+        const int tx = lt % cam.tiles_x, ty = lt / cam.tiles_x;
+        const int px = tx * TS + 8 * (wb % (TS / 8)) + (lane & 7), py = ty * TS + 4 * (wb / (TS / 8)) + (lane >> 3);
+        const bool inside = px < cam.W && py < cam.H;
+        const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
+        const int2 rg = checked_range(a.ranges, t, P.pair_cap, a.st);
+        const int64_t vbase = (int64_t)view * P.N;
+        // VAR instances carry the variants (renormalised Top-K, spherical-harmonic
+        // item colours, low-pass filter), read from the parameters
+        const float* __restrict__ rgbv = a.rgb + (VAR && P.color_sh ? 3 * vbase : 0);
+        const int64_t pix = cam.pix_off + (int64_t)py * cam.W + px;
+        const uint32_t* list = a.list + rg.x;
+        const uint32_t* masks = a.masks + rg.x;
+        float* grows = a.grad_item + vbase * GRAD_STRIDE;  // this view's gradient rows
+
+        int nstop = 0;
+        float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
+        int kk = -1, next_pos = -1;
+        float next_dot = 0.0f;
+        // a selected surfel adds rn_a * dot + rn_b to what its weight multiplies:
+        // the dot itself, or (dot - F.dL/dF) / W for the renormalised variant
+        float rn_a = 1.0f, rn_b = 0.0f;
+        if (inside) {
+            nstop = min(a.saved_nstop[pix], rg.y - rg.x);
+            T = a.out_T[pix];
+            gr = a.d_rgb[3 * pix];
+            gg = a.d_rgb[3 * pix + 1];
+            gb = a.d_rgb[3 * pix + 2];
+            Sh = P.bg[0] * gr + P.bg[1] * gg + P.bg[2] * gb + (a.d_T ? a.d_T[pix] : 0.0f);
+            for (kk = K - 1; kk >= 0; --kk)
+                if (a.saved_pos[pix * K + kk] >= 0) break;
+            if (kk >= 0) {
+                next_pos = a.saved_pos[pix * K + kk];
+                next_dot = a.dots[pix * K + kk];
+            }
+            if (VAR && P.renorm) {  // entries 0..kk are the selected ones, front to back
+                float ws = 0.0f, wd = 0.0f;
+                for (int k2 = 0; k2 <= kk; ++k2) {
+                    const float wv = a.saved_w[pix * K + k2];
+                    ws += wv;
+                    wd = fmaf(wv, a.dots[pix * K + k2], wd);
+                }
+                rn_a = ws > 0.0f ? 1.0f / ws : 0.0f;
+                rn_b = -wd * rn_a * rn_a;
+            }
+        }
+        const int L = __reduce_max_sync(ALL, nstop);
+
+        // one chunk's records and gradient slots, and the lane mask of those the warp meets
+        auto stage = [&](int buf, const ListEntry& e) {
+            const int64_t sp = (int64_t)e.item - vbase;
+            if ((e.mask & wbit) && FSS_CHECKED(sp >= 0 && sp < P.N)) cp_async4(&G.slot[buf][lane], a.splat_slot + sp);
+            return stage_chunk(G.st[buf], e, wbit, a.rec, rgbv, vbase, P.N, a.st);
+        };
+        // chunk b0 is worked on while the one before it is copied and the list entries of the next are read
+        int b0 = ((L - 1) >> 5) << 5;  // (L = 0: the loop does not run)
+        ListEntry e1 = list_entry(list, masks, b0 + lane, L);
+        uint32_t word = stage((b0 >> 5) & 1, e1);
+        e1 = list_entry(list, masks, b0 - 32 + lane, L);
+        for (; b0 >= 0 && L > 0; b0 -= 32) {
+            const int buf = (b0 >> 5) & 1;
+            const WarpStage& S = G.st[buf];
+            const uint32_t next = stage(buf ^ 1, e1);
+            e1 = list_entry(list, masks, b0 - 64 + lane, L);
+            cp_async_wait_prev();  // this chunk's copies
+            __syncwarp();
+            for (uint32_t bits = word; bits != 0u; bits ^= 0x80000000u >> __clz(bits)) {
+                const int j = 31 - __clz(bits), pos = b0 + j;
+                float g[VAR ? 16 : 13];
+#pragma unroll
+                for (int k = 0; k < (VAR ? 16 : 13); ++k) g[k] = 0.0f;
+                bool contrib = false;
+                Hit h;
+                const float4 oc = S.oc[j];
+                if (pos < nstop &&
+                    eval_splat<VAR>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf, P.alpha_min, cam.near_plane, h, P.lowpass)) {
+                    contrib = true;
+                    const float alpha = fminf(h.alpha_raw, P.alpha_max);
+                    const float Tj = T * rcp_approx(1.0f - alpha);
+                    const float w = alpha * Tj;
+                    float s = oc.y * gr + oc.z * gg + oc.w * gb;
+                    if (pos == next_pos) {
+                        s += VAR ? fmaf(next_dot, rn_a, rn_b) : next_dot;
+                        --kk;
+                        next_pos = kk >= 0 ? a.saved_pos[pix * K + kk] : -1;
+                        next_dot = kk >= 0 ? a.dots[pix * K + kk] : 0.0f;
+                    }
+                    const float dal = Tj * (s - Sh);
+                    Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
+                    g[10] = w * gr;
+                    g[11] = w * gg;
+                    g[12] = w * gb;
+                    if (h.alpha_raw < P.alpha_max) {
+                        g[9] = dal * h.G;
+                        const float drho = -0.5f * alpha * dal;
+                        if (VAR && h.scr) {  // low-pass screen term: rho = 2 |x - c|^2, d rho / d c = -4 (X, Y)
+                            g[VAR ? 13 : 0] = -4.0f * h.X * drho;
+                            g[VAR ? 14 : 0] = -4.0f * h.Y * drho;
+                        } else {
+                            const float du = 2.0f * h.u * drho, dv = 2.0f * h.v * drho;
+                            const float gc0 = du * h.inv, gc1 = dv * h.inv, gc2 = -(du * h.u + dv * h.v) * h.inv;
+                            g[0] = gc0 * h.X; g[1] = gc0 * h.Y; g[2] = gc0;
+                            g[3] = gc1 * h.X; g[4] = gc1 * h.Y; g[5] = gc1;
+                            g[6] = gc2 * h.X; g[7] = gc2 * h.Y; g[8] = gc2;
+                        }
+                    }
+                    T = Tj;
+                }
+                if (__any_sync(ALL, contrib)) {
+                    if constexpr (VAR) reduce_scatter<16>(g);  // lane l holds value l >> 1
+                    else reduce_scatter13(g);
+                    const int slot = G.slot[buf][j];
+                    if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13) && in_bounds(a.st, SITE_SLOT, slot, P.N))
+                        atomicAdd(grows + (int64_t)slot * GRAD_STRIDE + (lane >> 1), g[0]);
+                }
+            }
+            word = next;
+            __syncwarp();  // every lane has read this half before the next copies into it
+        }
+        cp_async_wait_all();
+        __syncwarp();  // before the warp's next block
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -959,31 +1123,50 @@ cudaError_t launch_feat(const Cams& cams, const RParams& P, const BwdArgs& a, cu
     }
 }
 
-template <int TS, bool FULL, int CMAX, typename FT, bool VAR = false>
-cudaError_t launch_geo_one(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
-    constexpr int NB = FULL ? FBATCH : BB;
-    const size_t smem = (size_t)NB * (4 * 16 + 8) + (size_t)NB * 16 * 4 + (FULL ? (size_t)NB * P.C * 8 : 0);  // staging, masks, partials, rows
-    cudaError_t e = set_smem((const void*)k_bwd_geo<TS, FULL, CMAX, FT, VAR>, smem);
+template <int TS, int CMAX, typename FT, bool VAR>
+cudaError_t launch_geo_full(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
+    constexpr int NB = FBATCH;
+    const size_t smem = (size_t)NB * (4 * 16 + 8) + (size_t)NB * 16 * 4 + (size_t)NB * P.C * 8;  // staging, masks, partials, rows
+    cudaError_t e = set_smem((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR>, smem);
     if (e != cudaSuccess) return e;
     int grid = cams.total_tiles;
-    if (a.persistent && (e = persistent_grid((const void*)k_bwd_geo<TS, FULL, CMAX, FT, VAR>, TS * TS, smem, grid)) !=
-                            cudaSuccess)
+    if (a.persistent &&
+        (e = persistent_grid((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR>, TS * TS, smem, grid)) != cudaSuccess)
         return e;
-    k_bwd_geo<TS, FULL, CMAX, FT, VAR><<<grid, TS * TS, smem, s>>>(cams, P, a);
+    k_bwd_geo_full<TS, CMAX, FT, VAR><<<grid, TS * TS, smem, s>>>(cams, P, a);
     e = cudaGetLastError();
     if (e == cudaSuccess) kernel_mark(s);
     return e;
+}
+
+template <int TS>
+cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
+    constexpr int NT = TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS, PARTS = TS * TS / NT;
+    auto go = [&](auto kern) {
+        int64_t units = (int64_t)cams.total_tiles * PARTS;
+        if (a.persistent) {
+            int wave = (int)std::min<int64_t>(units, INT_MAX);
+            const cudaError_t e = persistent_grid((const void*)kern, NT, 0, wave);
+            if (e != cudaSuccess) return e;
+            units = wave;
+        }
+        kern<<<(unsigned)units, NT, 0, s>>>(cams, P, a);
+        const cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) kernel_mark(s);
+        return e;
+    };
+    return P.renorm || P.color_sh || P.lowpass ? go(k_bwd_geo_topk<TS, true>) : go(k_bwd_geo_topk<TS, false>);
 }
 
 template <int TS, typename FT>
 cudaError_t launch_geo(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
     // the variants (renormalised Top-K, spherical-harmonic colours, low-pass
     // filter) have their own instances: no cost on the plain paths
-    const bool var = P.renorm || P.color_sh || P.lowpass;
-    if (P.K > 0) return var ? launch_geo_one<TS, false, 4, FT, true>(cams, P, a, s) : launch_geo_one<TS, false, 4, FT>(cams, P, a, s);
-    if (P.C <= 32) return var ? launch_geo_one<TS, true, 32, FT, true>(cams, P, a, s) : launch_geo_one<TS, true, 32, FT>(cams, P, a, s);
-    if (P.C <= 64) return var ? launch_geo_one<TS, true, 64, FT, true>(cams, P, a, s) : launch_geo_one<TS, true, 64, FT>(cams, P, a, s);
-    return var ? launch_geo_one<TS, true, 128, FT, true>(cams, P, a, s) : launch_geo_one<TS, true, 128, FT>(cams, P, a, s);
+    if (P.K > 0) return launch_geo_topk<TS>(cams, P, a, s);
+    const bool var = P.color_sh || P.lowpass;
+    if (P.C <= 32) return var ? launch_geo_full<TS, 32, FT, true>(cams, P, a, s) : launch_geo_full<TS, 32, FT, false>(cams, P, a, s);
+    if (P.C <= 64) return var ? launch_geo_full<TS, 64, FT, true>(cams, P, a, s) : launch_geo_full<TS, 64, FT, false>(cams, P, a, s);
+    return var ? launch_geo_full<TS, 128, FT, true>(cams, P, a, s) : launch_geo_full<TS, 128, FT, false>(cams, P, a, s);
 }
 
 template <typename FT>
