@@ -57,6 +57,15 @@ namespace fss {
 // weight is always slot KCAP - 1.  With the first-K selection the K slots
 // after the padding take the first K contributors in order.
 //
+// PAIR: the intersections of two surfels do not depend on each other, so the
+// sets of 4 and 16 slots, which have the registers for it, start them together
+// (1.2M surfels, 1280 x 720: K = 3 335 -> 327 us, K = 12 520 -> 488; 3,000 in
+// 100 x 90: 97 -> 90 and 103 -> 97).  With 8 slots the 64 registers that 32
+// resident warps leave make it slower (406 -> 427 us).
+// Sets of 9 to 16 entries take 123 registers, 16 warps per SM, and are still
+// ahead of the set in shared memory (render_topk_wide.cuh) throughout: K = 12
+// above 488 us against 490, K = 16 with C = 48 561 / 630, small scenes 97 / 119.
+//
 // CTAs: TOPK_THREADS threads (parts of a tile), so that a block's registers
 // are free for the next one soon after it ends; the SORT instances keep a
 // tile's warps together, which sort its list first.
@@ -68,16 +77,19 @@ constexpr int topk_threads() {
 // shared memory of one warp: the two staging halves, whose place the selected
 // entries (32 rows of KCAP + 1 pairs) take afterwards, and (AUX) the normals
 // and argmax keys
-constexpr size_t topk_warp_smem(bool aux) { return 2 * sizeof(WarpStage) + (aux ? 32 * (16 + 8) : 0); }
+constexpr size_t topk_warp_smem(int kcap, bool aux) {
+    const size_t stage = 2 * sizeof(WarpStage), sel = (size_t)32 * (kcap + 1) * 8 + 128;
+    return (sel > stage ? sel : stage) + (aux ? 32 * (16 + 8) : 0);
+}
 
 template <int TS, int KCAP, typename FT, bool FRONT, bool AUX, bool LOSS = false, bool SORT = false>
-__global__ void __launch_bounds__(topk_threads<TS, SORT>(), 1024 / topk_threads<TS, SORT>()) k_render_topk(
+__global__ void __launch_bounds__(topk_threads<TS, SORT>(), (KCAP <= 8 ? 1024 : 512) / topk_threads<TS, SORT>()) k_render_topk(
     const __grid_constant__ Cams cams, const __grid_constant__ RParams P, const FwdArgs a,
     const __grid_constant__ AuxOut x) {
     constexpr int NT = topk_threads<TS, SORT>(), NW = NT / 32, PARTS = TS * TS / NT;
+    constexpr bool PAIR = KCAP != 8;  // two surfels' intersections at a time (see above)
     constexpr int ROW = KCAP + 1;  // padded row of a pixel's selected entries (bank conflicts)
     constexpr unsigned ALL = 0xffffffffu;
-    static_assert(KCAP <= 8 && 32 * ROW * 8 + 128 <= 2 * sizeof(WarpStage), "the entries fit the staging halves");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_work;
     __shared__ float s_loss[LOSS ? NW : 1];  // LOSS: the warps' sums of a tile (part)
@@ -85,10 +97,10 @@ __global__ void __launch_bounds__(topk_threads<TS, SORT>(), 1024 / topk_threads<
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (a.st->err) return;
-    unsigned char* base = smem + warp * topk_warp_smem(AUX);
+    unsigned char* base = smem + warp * topk_warp_smem(KCAP, AUX);
     WarpStage* s_st = reinterpret_cast<WarpStage*>(base);     // [2]
-    float4* s_nrm = reinterpret_cast<float4*>(s_st + 2);      // AUX: [32] facing normals, centre depths
-    unsigned long long* s_lab = reinterpret_cast<unsigned long long*>(s_nrm + 32);  // AUX: [32] argmax keys
+    float4* s_nrm = reinterpret_cast<float4*>(base + topk_warp_smem(KCAP, false));  // AUX: [32] facing normals, centre depths
+    unsigned long long* s_lab = reinterpret_cast<unsigned long long*>(s_nrm + 32);    // AUX: [32] argmax keys
     int2* s_sel = reinterpret_cast<int2*>(base);              // phase 2: [32][ROW] (list position, then surfel id; weight)
     int32_t* s_n = reinterpret_cast<int32_t*>(s_sel + 32 * ROW);  // [32] selected entries
     const int K = P.K;
@@ -176,56 +188,78 @@ __global__ void __launch_bounds__(topk_threads<TS, SORT>(), 1024 / topk_threads<
                 }
                 __syncwarp();
             }
+            // one surfel: true when the pixel stops
+            auto composite = [&](int j, const float4& oc, const Hit& h) {
+                const float alpha = fminf(h.alpha_raw, P.alpha_max);
+                const float Tn = T * (1.0f - alpha);
+                if (Tn < P.T_min) return true;
+                const float w = alpha * T;
+                cr = fmaf(w, oc.y, cr);
+                cg = fmaf(w, oc.z, cg);
+                cb = fmaf(w, oc.w, cb);
+                ++n_contrib;
+                if (AUX) {
+                    const float4 nv = s_nrm[j];
+                    const float zh = h.scr ? nv.w : S.r2[j].w * h.inv;  // hit depth, as in the near-plane test
+                    zs = fmaf(w, zh, zs);
+                    nx = fmaf(w, nv.x, nx);
+                    ny = fmaf(w, nv.y, ny);
+                    nz = fmaf(w, nv.z, nz);
+                    if (!med && Tn < 0.5f) { zmed = zh; med = true; }
+                }
+                if (FRONT) {
+                    // the first K contributors, in the K slots after the padding
+                    if (n_sel < K) {
+                        const int slot = KCAP - K + n_sel;
+#pragma unroll
+                        for (int k = 0; k < KCAP; ++k) {
+                            hw[k] = k == slot ? w : hw[k];
+                            hp[k] = k == slot ? b0 + j : hp[k];
+                        }
+                        ++n_sel;
+                    }
+                } else if (w > hw[KCAP - 1]) {
+#pragma unroll
+                    for (int k = KCAP - 1; k >= 0; --k) {
+                        const bool here = w > hw[k];  // w belongs in this slot or in front of it
+                        const bool above = k > 0 && w > hw[k > 0 ? k - 1 : 0];
+                        hp[k] = here ? (above ? hp[k > 0 ? k - 1 : 0] : b0 + j) : hp[k];
+                        hw[k] = k > 0 ? fmaxf(hw[k], fminf(hw[k > 0 ? k - 1 : 0], w)) : fmaxf(hw[0], w);
+                    }
+                }
+                T = Tn;
+                last = b0 + j;
+                return P.stop_rule == FSS_STOP_EXACT_TOPK && (FRONT ? n_sel == K : P.alpha_max * T <= hw[KCAP - 1]);
+            };
             if (!done) {
-                for (uint32_t bits = word; bits != 0u; bits &= bits - 1u) {
-                    const int j = __ffs(bits) - 1;
-                    ++n_eval;
-                    Hit h;
-                    const float4 oc = S.oc[j];
-                    if (!eval_splat<AUX>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf, P.alpha_min, cam.near_plane, h, P.lowpass))
-                        continue;
-                    const float alpha = fminf(h.alpha_raw, P.alpha_max);
-                    const float Tn = T * (1.0f - alpha);
-                    if (Tn < P.T_min) { done = true; break; }
-                    const float w = alpha * T;
-                    cr = fmaf(w, oc.y, cr);
-                    cg = fmaf(w, oc.z, cg);
-                    cb = fmaf(w, oc.w, cb);
-                    ++n_contrib;
-                    if (AUX) {
-                        const float4 nv = s_nrm[j];
-                        const float zh = h.scr ? nv.w : S.r2[j].w * h.inv;  // hit depth, as in the near-plane test
-                        zs = fmaf(w, zh, zs);
-                        nx = fmaf(w, nv.x, nx);
-                        ny = fmaf(w, nv.y, ny);
-                        nz = fmaf(w, nv.z, nz);
-                        if (!med && Tn < 0.5f) { zmed = zh; med = true; }
+                if constexpr (PAIR) {
+                    for (uint32_t bits = word; bits != 0u;) {
+                        const int j0 = __ffs(bits) - 1;
+                        bits &= bits - 1u;
+                        const bool two = bits != 0u;
+                        const int j1 = two ? __ffs(bits) - 1 : j0;
+                        bits &= bits - 1u;
+                        Hit h0, h1;
+                        const bool hit0 = eval_splat<AUX>(S.r0[j0], S.r1[j0], S.r2[j0], S.oc[j0].x, pxf, pyf, P.alpha_min,
+                                                          cam.near_plane, h0, P.lowpass);
+                        const bool hit1 = eval_splat<AUX>(S.r0[j1], S.r1[j1], S.r2[j1], S.oc[j1].x, pxf, pyf, P.alpha_min,
+                                                          cam.near_plane, h1, P.lowpass) && two;
+                        ++n_eval;
+                        if (hit0 && composite(j0, S.oc[j0], h0)) { done = true; break; }
+                        n_eval += two ? 1u : 0u;
+                        if (hit1 && composite(j1, S.oc[j1], h1)) { done = true; break; }
                     }
-                    if (FRONT) {
-                        // the first K contributors, in the K slots after the padding
-                        if (n_sel < K) {
-                            const int slot = KCAP - K + n_sel;
-#pragma unroll
-                            for (int k = 0; k < KCAP; ++k) {
-                                hw[k] = k == slot ? w : hw[k];
-                                hp[k] = k == slot ? b0 + j : hp[k];
-                            }
-                            ++n_sel;
+                } else {
+                    for (uint32_t bits = word; bits != 0u; bits &= bits - 1u) {
+                        const int j = __ffs(bits) - 1;
+                        ++n_eval;
+                        Hit h;
+                        const float4 oc = S.oc[j];
+                        if (eval_splat<AUX>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf, P.alpha_min, cam.near_plane, h, P.lowpass) &&
+                            composite(j, oc, h)) {
+                            done = true;
+                            break;
                         }
-                    } else if (w > hw[KCAP - 1]) {
-#pragma unroll
-                        for (int k = KCAP - 1; k >= 0; --k) {
-                            const bool here = w > hw[k];                     // x goes to this slot or a later one's front
-                            const bool above = k > 0 && w > hw[k > 0 ? k - 1 : 0];
-                            hp[k] = here ? (above ? hp[k > 0 ? k - 1 : 0] : b0 + j) : hp[k];
-                            hw[k] = k > 0 ? fmaxf(hw[k], fminf(hw[k > 0 ? k - 1 : 0], w)) : fmaxf(hw[0], w);
-                        }
-                    }
-                    T = Tn;
-                    last = b0 + j;
-                    if (P.stop_rule == FSS_STOP_EXACT_TOPK && (FRONT ? n_sel == K : P.alpha_max * T <= hw[KCAP - 1])) {
-                        done = true;
-                        break;
                     }
                 }
             }
@@ -415,22 +449,24 @@ cudaError_t launch_topk(const Cams& cams, const RParams& P, const FwdArgs& a, co
                         cudaStream_t s) {
     constexpr int NT = topk_threads<TS, false>(), PARTS = TS * TS / NT;
     const bool aux = x.any() || P.lowpass;  // the variant instances also carry the low-pass filter
-    const size_t smem = NT / 32 * topk_warp_smem(aux);
+    auto smem = [aux](int kcap) { return NT / 32 * topk_warp_smem(kcap, aux); };
     // the fused loss (and sort): the plain selection with K <= 8, no sensor outputs (checked by the caller)
     if (x.loss.loss && x.sort.list)
         return launch_tiles(k_render_topk<TS, 8, FT, false, false, true, true>, TS * TS,
-                            std::max(TS * TS / 32 * topk_warp_smem(false), SORT_SMEM_BYTES), cams, P, a, x, num_sms, s);
+                            std::max(TS * TS / 32 * topk_warp_smem(8, false), SORT_SMEM_BYTES), cams, P, a, x, num_sms, s);
     if (x.loss.loss)
-        return launch_tiles(k_render_topk<TS, 8, FT, false, false, true>, NT, smem, cams, P, a, x, num_sms, s, PARTS);
-    // sets of more than eight entries live in shared memory (render_topk_wide.cuh):
-    // in registers K = 9..16 take 112 registers and K = 32 220
-    if (P.K > 8) return launch_topk_wide<TS, FT>(cams, P, a, x, num_sms, s);
-    auto go = [&](auto kern) { return launch_tiles(kern, NT, smem, cams, P, a, x, num_sms, s, PARTS); };
+        return launch_tiles(k_render_topk<TS, 8, FT, false, false, true>, NT, smem(8), cams, P, a, x, num_sms, s, PARTS);
+    // larger sets live in shared memory (render_topk_wide.cuh): those of more than
+    // 16 entries, and more than 8 for the variants, which need the registers
+    const bool plain = !aux && P.select != FSS_SELECT_FRONT;
+    if (P.K > (plain ? 16 : 8)) return launch_topk_wide<TS, FT>(cams, P, a, x, num_sms, s);
+    auto go = [&](auto kern, int kcap = 8) { return launch_tiles(kern, NT, smem(kcap), cams, P, a, x, num_sms, s, PARTS); };
     if (P.select == FSS_SELECT_FRONT)
         return aux ? go(k_render_topk<TS, 8, FT, true, true>) : go(k_render_topk<TS, 8, FT, true, false>);
     if (aux) return go(k_render_topk<TS, 8, FT, false, true>);
-    if (P.K <= 4) return go(k_render_topk<TS, 4, FT, false, false>);
-    return go(k_render_topk<TS, 8, FT, false, false>);
+    if (P.K <= 4) return go(k_render_topk<TS, 4, FT, false, false>, 4);
+    if (P.K <= 8) return go(k_render_topk<TS, 8, FT, false, false>);
+    return go(k_render_topk<TS, 16, FT, false, false>, 16);
 }
 
 template <typename FT>

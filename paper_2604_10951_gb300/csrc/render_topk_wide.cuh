@@ -1,4 +1,4 @@
-// Top-K forward render for K > 8 (included by one translation unit per
+// Top-K forward render for K > 16 (variants: K > 8; included by one translation unit per
 // feature type): the traversal, selection rule and outputs of render_topk.cuh,
 // with the K-set of a pixel in shared memory instead of registers.
 //

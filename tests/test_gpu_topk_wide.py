@@ -1,4 +1,4 @@
-"""GPU parity of the Top-K forward for K > 8 (the K-set in shared memory):
+"""GPU parity of the Top-K forward for K > 8 (register sets to 16, then shared memory):
 scenes of faint surfels, where most pixels meet more than K contributors and
 slots are refilled, over K at and beside the slot groups of eight, the tile
 sizes, a ragged image and the variants; and the tie rule (equal weights: the
