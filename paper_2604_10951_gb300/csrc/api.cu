@@ -390,14 +390,11 @@ fss_status fss_project_bin(const fss_params* params, const fss_camera* cams, int
     if ((e = arm_guards(ctx, st)) != cudaSuccess) return cuda_fail(e, "memset canaries");
     const int sms = num_sms_current();
     Status* stp = ctx.at<Status>(REG_STATUS);
-    const int64_t items = ctx.P.n_items;
-    const int64_t blocks = std::max<int64_t>(1, (items + 1023) / 1024);  // PROJ_ITEMS items per CTA
-    k_project<<<(unsigned)blocks, 256, 0, st>>>(ctx.cams, ctx.P, means, scales, quats, opac, ctx.at<float4>(REG_REC),
-                                               ctx.at<BinRec>(REG_BINREC), ctx.at<uint32_t>(REG_COUNT),
-                                               ctx.at<uint32_t>(REG_TILECNT), ctx.at<uint32_t>(REG_VIS),
-                                               ctx.at<uint32_t>(REG_WIDE), ctx.at<uint32_t>(REG_UNB),
-                                               ctx.at<int32_t>(REG_SLOT), ctx.at<int32_t>(REG_SLOT_SURF), stp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "k_project");
+    e = launch_project(ctx.cams, ctx.P, means, scales, quats, opac, ctx.at<float4>(REG_REC), ctx.at<BinRec>(REG_BINREC),
+                       ctx.at<uint32_t>(REG_COUNT), ctx.at<uint32_t>(REG_TILECNT), ctx.at<uint32_t>(REG_VIS),
+                       ctx.at<uint32_t>(REG_WIDE), ctx.at<uint32_t>(REG_UNB), ctx.at<int32_t>(REG_SLOT),
+                       ctx.at<int32_t>(REG_SLOT_SURF), stp, sms, st);
+    if (e != cudaSuccess) return cuda_fail(e, "k_project");
     kernel_mark(st);
     // one resident wave: records run from the lowest threads up, tile emission
     // from the highest down, so both start at once; one CTA scans the tile

@@ -25,13 +25,11 @@ bool kernel_marks_armed();
 // failed): the caller then stays in `s`.
 bool side_stream(cudaStream_t s, cudaStream_t& side, cudaEvent_t& fork, cudaEvent_t& join);
 
-__global__ void k_project(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
-                          const float* __restrict__ means, const float* __restrict__ scales,
-                          const float* __restrict__ quats, const float* __restrict__ opac, float4* __restrict__ rec,
-                          BinRec* __restrict__ binrec, uint32_t* __restrict__ count, uint32_t* __restrict__ tile_cnt,
-                          uint32_t* __restrict__ vis_list, uint32_t* __restrict__ wide_list,
-                          uint32_t* __restrict__ unb_list, int32_t* __restrict__ splat_slot,
-                          int32_t* __restrict__ slot_surf, Status* __restrict__ st);
+// projection and tile counts (k_project)
+cudaError_t launch_project(const Cams& cams, const RParams& P, const float* means, const float* scales, const float* quats,
+                           const float* opac, float4* rec, BinRec* binrec, uint32_t* count, uint32_t* tile_cnt,
+                           uint32_t* vis_list, uint32_t* wide_list, uint32_t* unb_list, int32_t* splat_slot,
+                           int32_t* slot_surf, Status* st, int num_sms, cudaStream_t stream);
 cudaError_t set_hold_scan(int hold);  // fss_test_hold_scan
 __global__ void k_emit(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
                        const BinRec* __restrict__ binrec, const uint32_t* __restrict__ vis_list,

@@ -19,6 +19,10 @@
 #include "fss_internal.cuh"
 #include "kernels.cuh"
 
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
 namespace fss {
 
 namespace {
@@ -375,24 +379,57 @@ __device__ __forceinline__ bool early_culls(const CamDev& cam, const RParams& P,
     return true;
 }
 
-constexpr int PROJ_ITEMS = 1024;  // items per CTA of k_project
+// A cheap superset of early_culls: true only for items that it culls.  The
+// depth and opacity tests are its own; the frustum test takes the largest
+// radius that an opacity of at most 1 can give (`rmax` times the larger scale:
+// a larger sphere's box contains the smaller one's), multiplies instead of
+// dividing, and leaves half a pixel and 1e-5 of the image coordinates for its
+// rounding.  Opacities above 1 and non-finite values go on to early_culls.
+__device__ __forceinline__ bool surely_culled(const CamDev& cam, const RParams& P, const CullIn& in, float rmax,
+                                              float mmax) {
+    float e[3], pc[3];
+    mvec(cam.R, in.pm, e);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) pc[i] = fa(e[i], cam.t[i]);
+    if (!(pc[2] > cam.near_plane) || !(in.o >= P.alpha_min)) return true;
+    const float r = fmaf(rmax, fmaxf(in.sc.x, in.sc.y), 1e-5f);
+    const float zlo = pc[2] - r, zhi = pc[2] + r;
+    const float sx = mmax + 1e-5f * (fabsf(cam.cx) + (float)cam.W), sy = mmax + 1e-5f * (fabsf(cam.cy) + (float)cam.H);
+    const float xa = pc[0] - r, xb = pc[0] + r, ya = pc[1] - r, yb = pc[1] + r;
+    const bool out = cam.fx * xb < -(cam.cx + sx) * (xb >= 0.0f ? zlo : zhi) ||
+                     cam.fx * xa > ((float)cam.W + sx - cam.cx) * (xa >= 0.0f ? zhi : zlo) ||
+                     cam.fy * yb < -(cam.cy + sy) * (yb >= 0.0f ? zlo : zhi) ||
+                     cam.fy * ya > ((float)cam.H + sy - cam.cy) * (ya >= 0.0f ? zhi : zlo);
+    return out && zlo > 0.0f && in.o <= 1.0f;
+}
+
 constexpr int PROJ_THREADS = 256;
 
 // ---------------------------------------------------------------------------
-// k_project: (view, surfel) items, PROJ_ITEMS per CTA
+// k_project: (view, surfel) items, PER * 256 per CTA
 //
-// Stage A runs the cheap culls (depth, opacity, frustum) one thread per item
-// and queues the survivors in shared memory; stage B runs the rest of the
-// chain one thread per survivor, so the few visible surfels of a view fill
-// whole warps instead of one lane in each.  A visible item with a bounded conic counts
-// its tiles (fire-and-forget adds into the per-tile counters, cleared by the
-// host call before this kernel) and is appended to the narrow list, or to
-// the wide list when it spans more than WIDE_TILES tiles; an unbounded item
-// goes to its view's list instead (every tile of the view includes it).
-// Appends and gradient-slot claims are aggregated per warp.
+// Stage A drops the items that the cheap superset of the culls is sure about,
+// one thread per item, and queues the rest in shared memory; stage B runs the
+// exact culls and the chain one thread per queued item, so the few visible
+// surfels of a view fill whole warps instead of one lane in each.  A visible
+// item with a bounded conic counts its tiles (fire-and-forget adds into the
+// per-tile counters, cleared by the host call before this kernel) and is
+// appended to the narrow list, or to the wide list when it spans more than
+// WIDE_TILES tiles; an unbounded item goes to its view's list instead (every
+// tile of the view includes it).  Appends and gradient-slot claims are
+// aggregated per warp.
+//
+// PER = 4 packs stage B well where most items are culled; PER = 1 spreads few
+// items over the SMs: below 1024 items per SM (1,000 surfels in a 128 x 128
+// frame: 66 -> 41 us for the whole forward, with PER = 4 62; 150k in a room 73
+// -> 69, 71; 300k 87 -> 89, 85).  Stage A is bound by the latency of its loads;
+// with the exact culls in it (a logarithm, a square root and four divisions per
+// item) 1.5M items took 50 us where this takes 42, and 12M items 279 / 220.
 // ---------------------------------------------------------------------------
 constexpr uint32_t WIDE_TILES = 32;
+constexpr int64_t PROJ_SPREAD = 1024;  // items per SM below which a CTA takes 256 of them
 
+template <int PER>
 __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
                                                  const float* __restrict__ means, const float* __restrict__ scales,
                                                  const float* __restrict__ quats, const float* __restrict__ opac,
@@ -400,7 +437,9 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
                                                  uint32_t* __restrict__ count, uint32_t* __restrict__ tile_cnt,
                                                  uint32_t* __restrict__ vis_list, uint32_t* __restrict__ wide_list,
                                                  uint32_t* __restrict__ unb_list, int32_t* __restrict__ splat_slot,
-                                                 int32_t* __restrict__ slot_surf, Status* __restrict__ st) {
+                                                 int32_t* __restrict__ slot_surf, Status* __restrict__ st, float rmax,
+                                                 float mmax) {
+    constexpr int PROJ_ITEMS = PER * PROJ_THREADS;
     __shared__ uint32_t s_q[PROJ_ITEMS];
     __shared__ int s_nq;
     __shared__ BinRec s_br[PROJ_THREADS];
@@ -412,10 +451,9 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     const int lane = threadIdx.x & 31;
     if (threadIdx.x == 0) s_nq = 0;
     __syncthreads();
-    // stage A: the cheap culls for PROJ_ITEMS items (each thread's items loaded
-    // together first); survivors queued in shared memory
+    // stage A: the superset of the culls for PROJ_ITEMS items (each thread's items
+    // loaded together first); the rest queued in shared memory
     const int64_t base = (int64_t)blockIdx.x * PROJ_ITEMS;
-    constexpr int PER = PROJ_ITEMS / PROJ_THREADS;
     CullIn in[PER];
     int vw[PER];
 #pragma unroll
@@ -431,11 +469,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     for (int i = 0; i < PER; ++i) {
         const int k = threadIdx.x + i * PROJ_THREADS;
         const int64_t it = base + k;
-        bool keep = false;
-        if (it < P.n_items) {
-            float pc[3], o;
-            keep = early_culls(cams.c[vw[i]], P, in[i], pc, o);
-        }
+        const bool keep = it < P.n_items && !surely_culled(cams.c[vw[i]], P, in[i], rmax, mmax);
         const unsigned m = __ballot_sync(0xffffffffu, keep);
         int b = 0;
         if (lane == 0 && m) b = atomicAdd(&s_nq, __popc(m));
@@ -444,7 +478,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     }
     __syncthreads();
     const int nq = s_nq;
-    // stage B: the whole chain for the survivors, packed densely into warps
+    // stage B: the whole chain for the queued items, packed densely into warps
     // (warp-uniform loop: the appends below use whole-warp ballots)
     for (int q0 = threadIdx.x & ~31; q0 < nq; q0 += blockDim.x) {
     const int64_t item = q0 + lane < nq ? base + s_q[q0 + lane] : P.n_items;
@@ -681,6 +715,25 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
         if (in_bounds(st, SITE_VIS_LIST, k, P.N)) unb_list[(int64_t)view * P.N + k] = (uint32_t)item;
     }
     }  // survivors
+}
+
+cudaError_t launch_project(const Cams& cams, const RParams& P, const float* means, const float* scales, const float* quats,
+                           const float* opac, float4* rec, BinRec* binrec, uint32_t* count, uint32_t* tile_cnt,
+                           uint32_t* vis_list, uint32_t* wide_list, uint32_t* unb_list, int32_t* splat_slot,
+                           int32_t* slot_surf, Status* st, int num_sms, cudaStream_t stream) {
+    // the largest binning radius per unit scale and screen margin of an opacity <= 1, widened (see surely_culled)
+    const double k2 = 2.0 * std::log(1.0 / (double)P.alpha_min) * 1.0009765625;
+    const float rmax = (float)(std::sqrt(std::max(k2, 0.0)) * 1.0015);
+    const float mmax = (float)(1.0 + (P.lowpass ? std::sqrt(std::max(k2, 0.0) * 0.5) * 1.0015 : 0.0));
+    auto go = [&](auto per) {
+        constexpr int PER = decltype(per)::value;
+        const int64_t blocks = std::max<int64_t>(1, (P.n_items + PER * PROJ_THREADS - 1) / (PER * PROJ_THREADS));
+        k_project<PER><<<(unsigned)blocks, PROJ_THREADS, 0, stream>>>(cams, P, means, scales, quats, opac, rec, binrec,
+                                                                    count, tile_cnt, vis_list, wide_list, unb_list,
+                                                                    splat_slot, slot_surf, st, rmax, mmax);
+        return cudaGetLastError();
+    };
+    return P.n_items < PROJ_SPREAD * num_sms ? go(std::integral_constant<int, 1>{}) : go(std::integral_constant<int, 4>{});
 }
 
 // ---------------------------------------------------------------------------
