@@ -862,7 +862,7 @@ __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
 }
 
 // ---------------------------------------------------------------------------
-// precise render record (see record_item_quad), written in double-float
+// precise render record (record_item), written in double-float
 //
 // The ray-splat solve u ~ adj(T') (x - xc, y - yc, 1) is evaluated per pixel
 // in binary32, but the adjugate itself is computed here in double-float from
@@ -875,86 +875,69 @@ __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
 // (unnormalised) rotation polynomial, so n2 * T = K [r_u Rv t_u', r_v Rv t_v',
 // n2 (Rv p + t)] needs no square root; its adjugate is n2^2 adj(T).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ df shfl_df(df v, int src) {
-    return {__shfl_sync(0xffffffffu, v.hi, src, 4), __shfl_sync(0xffffffffu, v.lo, src, 4)};
-}
-
-// One quad of lanes per item (j = lane & 3): lane j < 3 forms column j of the
-// shifted n2 T' (the two tangent columns and the centre column), the quad
-// exchanges the columns, and lane r < 3 forms adjugate row r; the operations
-// and their order are those of a single-thread evaluation, so the record
-// does not depend on the split.  Every lane of the warp must call this
-// (shuffles); `valid` false computes nothing that is stored.
-__device__ void record_item_quad(const Cams& cams, const RParams& P, const float* __restrict__ means,
-                                 const float* __restrict__ scales, const float* __restrict__ quats,
-                                 float4* __restrict__ rec, uint32_t item, bool valid) {
-    const int j = threadIdx.x & 3, q0 = (threadIdx.x & 31) & ~3;
+// One thread per item.  (A quad of lanes per item, one column each, formed the
+// rotation in every lane and exchanged the columns: 2.2 times the instructions,
+// MEASURED_REC)
+__device__ __forceinline__ void record_item(const Cams& cams, const RParams& P, const float* __restrict__ means,
+                                            const float* __restrict__ scales, const float* __restrict__ quats,
+                                            float4* __restrict__ rec, uint32_t item) {
     const int view = view_of_item(item, P.N);
     const int64_t s = (int64_t)item - (int64_t)view * P.N;
     const CamDev& cam = cams.c[view];
     float4* rr = rec + 4 * (size_t)item;
     const float xc = rr[0].w, yc = rr[1].w;
     const float4 q4 = __ldg(reinterpret_cast<const float4*>(quats) + s);
+    const float2 sc = __ldg(reinterpret_cast<const float2*>(scales) + s);
+    const float pm[3] = {__ldg(means + 3 * s), __ldg(means + 3 * s + 1), __ldg(means + 3 * s + 2)};
     const float qw = q4.x, qx = q4.y, qy = q4.z, qz = q4.w;
     const df ww = two_prod(qw, qw), xx = two_prod(qx, qx), yy = two_prod(qy, qy), zz = two_prod(qz, qz);
     const df n2 = dadd(dadd(ww, xx), dadd(yy, zz));
-    // column j of n2 T (camera frame, before the intrinsics): R t_u' r_u,
-    // R t_v' r_v or n2 (R p + t); straight-line code with selects, so the
-    // quad's lanes do not diverge
-    const df xy = two_prod(qx, qy), wz = two_prod(qw, qz), xz = two_prod(qx, qz), wy = two_prod(qw, qy);
-    const df yz = two_prod(qy, qz), wx = two_prod(qw, qx);
-    const df tu[3] = {dsub(dadd(ww, xx), dadd(yy, zz)), dmulf(dadd(xy, wz), 2.0f), dmulf(dsub(xz, wy), 2.0f)};
-    const df tv[3] = {dmulf(dsub(xy, wz), 2.0f), dsub(dadd(ww, yy), dadd(xx, zz)), dmulf(dadd(yz, wx), 2.0f)};
-    const df pm[3] = {dfrom(means[3 * s]), dfrom(means[3 * s + 1]), dfrom(means[3 * s + 2])};
-    df v[3], e[3], col[3];
+    df d[3][3];  // the columns of n2 T, shifted about (xc, yc)
 #pragma unroll
-    for (int i = 0; i < 3; ++i) v[i] = j == 0 ? tu[i] : (j == 1 ? tv[i] : pm[i]);
-    dmvec(cam.R, v, e);
-    const float sj = scales[2 * s + (j == 1 ? 1 : 0)];
+    for (int j = 0; j < 3; ++j) {
+        // column j of n2 T (camera frame, before the intrinsics): R t_u' r_u, R t_v' r_v or n2 (R p + t)
+        df v[3], col[3];
+        if (j == 0) {
+            v[0] = dsub(dadd(ww, xx), dadd(yy, zz));
+            v[1] = dmulf(dadd(two_prod(qx, qy), two_prod(qw, qz)), 2.0f);
+            v[2] = dmulf(dsub(two_prod(qx, qz), two_prod(qw, qy)), 2.0f);
+        } else if (j == 1) {
+            v[0] = dmulf(dsub(two_prod(qx, qy), two_prod(qw, qz)), 2.0f);
+            v[1] = dsub(dadd(ww, yy), dadd(xx, zz));
+            v[2] = dmulf(dadd(two_prod(qy, qz), two_prod(qw, qx)), 2.0f);
+        } else {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const df a = dmulf(e[i], sj), b = dmul(dadd(e[i], dfrom(cam.t[i])), n2);
-        col[i] = j < 2 ? a : b;
+            for (int i = 0; i < 3; ++i) v[i] = dfrom(pm[i]);
+        }
+        dmvec(cam.R, v, col);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            col[i] = j < 2 ? dmulf(col[i], j == 0 ? sc.x : sc.y) : dmul(dadd(col[i], dfrom(cam.t[i])), n2);
+        d[j][0] = dsub(dadd(dmulf(col[0], cam.fx), dmulf(col[2], cam.cx)), dmulf(col[2], xc));
+        d[j][1] = dsub(dadd(dmulf(col[1], cam.fy), dmulf(col[2], cam.cy)), dmulf(col[2], yc));
+        d[j][2] = col[2];
     }
-    // column j of n2 T, shifted about (xc, yc)
-    df dj[3];
-    {
-        const df cx = dadd(dmulf(col[0], cam.fx), dmulf(col[2], cam.cx));
-        const df cy = dadd(dmulf(col[1], cam.fy), dmulf(col[2], cam.cy));
-        dj[0] = dsub(cx, dmulf(col[2], xc));
-        dj[1] = dsub(cy, dmulf(col[2], yc));
-        dj[2] = col[2];
-    }
-    df d[3][3];
+    // adjugate rows m_j = d_{j+1} x d_{j+2}
+    df m[3][3];
+    dcross(d[1], d[2], m[0]);
+    dcross(d[2], d[0], m[1]);
+    dcross(d[0], d[1], m[2]);
+    float mx = 0.0f;
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+    for (int j = 0; j < 3; ++j)
 #pragma unroll
-        for (int i = 0; i < 3; ++i) d[c][i] = shfl_df(dj[i], q0 + c);
-    // adjugate row j: m_j = d_{j+1} x d_{j+2} (operands picked by selects: a
-    // dynamic index would put d in local memory)
-    const int r = j < 3 ? j : 0;
-    df da[3], db[3], m[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        da[i] = r == 0 ? d[1][i] : (r == 1 ? d[2][i] : d[0][i]);
-        db[i] = r == 0 ? d[2][i] : (r == 1 ? d[0][i] : d[1][i]);
-    }
-    dcross(da, db, m);
-    float mx = j < 3 ? fmaxf(fmaxf(fabsf(m[0].hi), fabsf(m[1].hi)), fabsf(m[2].hi)) : 0.0f;
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1, 4));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2, 4));
-    // lane 0: det(n2 T') from row 0
-    const df det = dadd(dadd(dmul(d[0][0], m[0]), dmul(d[0][1], m[1])), dmul(d[0][2], m[2]));
+        for (int i = 0; i < 3; ++i) mx = fmaxf(mx, fabsf(m[j][i].hi));
+    if (!(mx > 0.0f)) return;
+    const df det = dadd(dadd(dmul(d[0][0], m[0][0]), dmul(d[0][1], m[0][1])), dmul(d[0][2], m[0][2]));  // det(n2 T')
     int ex = 0;
-    if (mx > 0.0f) frexp32(mx, &ex);
+    frexp32(mx, &ex);
     // hit depth det(T') / c2: with M = 2^-ex n2^2 adj(T'), store 2^-ex det(n2 T') / n2
-    const float detr = __shfl_sync(0xffffffffu, ldexp32(fdv(det.hi, n2.hi), -ex), q0);
-    if (!valid || !(mx > 0.0f)) return;  // after the last shuffle: every lane took part
-    if (j < 3)
-        rr[j] = make_float4(ldexp32(m[0].hi, -ex), ldexp32(m[1].hi, -ex), ldexp32(m[2].hi, -ex),
+    const float detr = ldexp32(fdv(det.hi, n2.hi), -ex);
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        rr[j] = make_float4(ldexp32(m[j][0].hi, -ex), ldexp32(m[j][1].hi, -ex), ldexp32(m[j][2].hi, -ex),
                             j == 0 ? xc : (j == 1 ? yc : detr));
-    // total scale of M relative to adj(T' of the normalised surfel)
-    if (j == 0) rr[3].w = ldexp32(fm(n2.hi, n2.hi), -ex);
+    rr[3].w = ldexp32(fm(n2.hi, n2.hi), -ex);  // total scale of M relative to adj(T' of the normalised surfel)
 }
 
 constexpr int EMIT_BATCH = 8;
@@ -980,8 +963,8 @@ __device__ __forceinline__ void emit_batch(uint32_t* __restrict__ cursor, uint32
 //                 into ranges and emit cursors and publishes them (release
 //                 store of a flag); it never waits, so the others' bounded
 //                 wait for the flag ends however the CTAs are scheduled;
-//   records:      one quad of lanes per narrow, wide or unbounded item (they
-//                 need no ranges, so they run while the scan does);
+//   records:      one thread per narrow, wide or unbounded item (they need no
+//                 ranges, so they run while the scan does);
 //   narrow items: 32 per warp, their (item, outer line) units spread over
 //                 the lanes; each lane emits its line's tiles;
 //   wide items:   one warp per (item, outer line), lanes over the line's tiles;
@@ -1017,29 +1000,24 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Cams cams,
     const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
     uint32_t nunb = 0;
     for (int v = 0; v < cams.n; ++v) nunb += st->unb_cnt[v];
-    // render records of all visible items (narrow, wide, unbounded), one quad
-    // of lanes each, from the lowest threads up (warp-uniform loop)
+    // render records of all visible items (narrow, wide, unbounded), one thread
+    // each, from the lowest threads up
     const uint32_t nrec = nvis + nwide + nunb;
-    for (int64_t base = (gtid >> 5) * 8; base < nrec; base += (gstride >> 5) * 8) {
-        const int64_t ri = base + (lane >> 2);
-        const bool valid = ri < nrec;
+    for (int64_t ri = gtid; ri < nrec; ri += gstride) {
         uint32_t item = 0;
-        bool ok = valid && in_bounds(stw, SITE_VIS_LIST, ri, P.n_items);
-        if (ok) {
-            if (ri < nvis) {
-                item = vis_list[ri];
-            } else if (ri < (int64_t)nvis + nwide) {
-                item = wide_list[ri - nvis];
-            } else {
-                uint32_t k = (uint32_t)(ri - nvis - nwide);
-                int v = 0;
-                while (FSS_CHECKED(v < cams.n) && k >= st->unb_cnt[v]) k -= st->unb_cnt[v++];
-                ok = in_bounds(stw, SITE_VIS_LIST, v, cams.n) && in_bounds(stw, SITE_VIS_LIST, k, P.N);
-                item = ok ? unb_list[(int64_t)v * P.N + k] : 0u;
-            }
-            ok = ok && in_bounds(stw, SITE_ITEM, item, P.n_items);
+        if (!in_bounds(stw, SITE_VIS_LIST, ri, P.n_items)) break;
+        if (ri < nvis) {
+            item = vis_list[ri];
+        } else if (ri < (int64_t)nvis + nwide) {
+            item = wide_list[ri - nvis];
+        } else {
+            uint32_t k = (uint32_t)(ri - nvis - nwide);
+            int v = 0;
+            while (FSS_CHECKED(v < cams.n) && k >= st->unb_cnt[v]) k -= st->unb_cnt[v++];
+            if (!in_bounds(stw, SITE_VIS_LIST, v, cams.n) || !in_bounds(stw, SITE_VIS_LIST, k, P.N)) continue;
+            item = unb_list[(int64_t)v * P.N + k];
         }
-        record_item_quad(cams, P, means, scales, quats, rec, ok ? item : 0u, valid && ok);
+        if (in_bounds(stw, SITE_ITEM, item, P.n_items)) record_item(cams, P, means, scales, quats, rec, item);
     }
     // the emit cursors: published by the scanning CTA (bounded wait)
     if (threadIdx.x == 0) {
