@@ -424,8 +424,8 @@ fss_status fss_project_bin(const fss_params* params, const fss_camera* cams, int
 namespace {
 
 fss_status launch_sort(Ctx& ctx, cudaStream_t st) {
-    k_tile_sort<<<ctx.cams.total_tiles, SORT_THREADS, 0, st>>>(ctx.cams, ctx.P, ctx.at<float4>(REG_REC),
-                                                      ctx.at<BinRec>(REG_BINREC), ctx.at<int2>(REG_RANGES),
+    k_tile_sort<<<ctx.cams.total_tiles, SORT_THREADS, 0, st>>>(ctx.cams, ctx.P, ctx.at<BinRec>(REG_BINREC),
+                                                      ctx.at<int2>(REG_RANGES),
                                                       ctx.at<uint32_t>(REG_LIST), ctx.at<uint32_t>(REG_UNB),
                                                       ctx.at<uint64_t>(REG_SORTTMP), ctx.at<uint32_t>(REG_MASK),
                                                       ctx.at<Status>(REG_STATUS));

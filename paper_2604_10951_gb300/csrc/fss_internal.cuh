@@ -79,7 +79,8 @@ struct alignas(16) BinRec {
     int16_t tx0, tx1, ty0, ty1;  // outer tile rectangle of the bin mode
     int32_t flags;           // BR_VISIBLE | BR_UNBOUNDED | BR_ELL | BR_LOWPASS
     float rd2;               // low-pass filter: screen disc radius^2 (pixels^2)
-    int32_t pad[2];
+    float z;                 // camera depth of the centre (the sort key)
+    int32_t pad;
 };
 static_assert(sizeof(BinRec) == 80, "BinRec layout");
 // BR_ELL: the cutoff ellipse has pixels (always set without the low-pass

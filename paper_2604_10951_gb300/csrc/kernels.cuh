@@ -39,7 +39,7 @@ __global__ void k_emit(const __grid_constant__ Cams cams, const __grid_constant_
                        const float* __restrict__ quats, float4* __restrict__ rec, Status* __restrict__ st,
                        int max_lines);
 __global__ void k_tile_sort(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
-                            const float4* __restrict__ rec, const BinRec* __restrict__ binrec,
+                            const BinRec* __restrict__ binrec,
                             const int2* __restrict__ ranges, uint32_t* __restrict__ list,
                             const uint32_t* __restrict__ unb_list, uint64_t* __restrict__ scratch,
                             uint32_t* __restrict__ masks, const Status* __restrict__ st);

@@ -125,10 +125,8 @@ __global__ void __launch_bounds__(topk_threads<TS, SORT>(), (KCAP <= 8 ? 1024 : 
         const int t = cams.tile_order ? cams.tile_order[u / PARTS] : u / PARTS;
         if constexpr (SORT) {  // this tile's depth sort first, in the staging area
             __syncthreads();   // (the previous tile's last reads of the area)
-            sort_tile(cams, P, a.rec, x.sort.binrec, a.ranges, x.sort.list, x.sort.unb_list, x.sort.scratch,
-                      x.sort.masks, a.st, t, reinterpret_cast<uint64_t*>(smem),
-                      reinterpret_cast<uint32_t*>(smem + (size_t)SORT_CAP * 8),
-                      reinterpret_cast<uint16_t*>(smem + (size_t)SORT_CAP * 12));
+            sort_tile(cams, P, x.sort.binrec, a.ranges, x.sort.list, x.sort.unb_list, x.sort.scratch,
+                      x.sort.masks, a.st, t, smem);
             __syncthreads();  // the sorted list and masks (global, written by this CTA) before staging
         }
         const int wb = (u % PARTS) * NW + warp;  // this warp's block of the tile
