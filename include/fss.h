@@ -435,9 +435,9 @@ const char *fss_last_error(void);
  *   boxes, flags); 3 tile count per item (uint32); 4 tile ranges
  *   (int32 [tiles, 2]); 5 tile lists (uint32 item ids, sorted by fss_sort);
  *   6 counters (uint64 [8], inside the status block: evaluations,
- *   contributions); 7 per-tile pair counts, then emission cursors (uint32,
- *   one per 32-byte sector);
- *   8 sort scratch (2 x uint64 per pair); 9 geometric gradient rows
+ *   contributions); 7 per-tile pair counts, then list places (uint32, one
+ *   32-byte sector per tile: narrow items, wide items);
+ *   8 sort scratch (2 x uint64 per pair; during binning the pair buffer); 9 geometric gradient rows
  *   (float [views, N, 16]); 10 feature gradient accumulators (float [N, C]);
  *   11 per-(pixel, k) dot products (float [pixels, K]); 12 visible item
  *   list; 13 unbounded items per view; 14 gradient slot per surfel (int32,

@@ -104,7 +104,7 @@ struct Status {
     uint32_t scan_done;    // ... and sets this (release) once the ranges and cursors are written
     uint32_t unb_cnt[FSS_MAX_CAMS];  // unbounded items per view
     uint32_t bounds_site;            // check build: first failed index check (BoundsSite), else 0
-    uint32_t pad4;
+    uint32_t npair;                  // (tile, slot, item) triples of narrow items written by k_project
     int64_t bounds_index;            // ... and the index it refused
 };
 enum { ERR_CAPACITY = 1, ERR_TIMEOUT = 2, ERR_BOUNDS = 4 };
@@ -169,9 +169,11 @@ constexpr uint32_t GUARD_WORD = 0xA5A5A5A5u;
 // ---------------------------------------------------------------------------
 // workspace layout (host computed, identical for every call of a frame)
 // ---------------------------------------------------------------------------
-// Per-tile pair counters (the emit cursors after the scan) sit one 32-byte
-// sector apart: every pair of the frame adds to one of them, and packed 32
-// to an L2 line the adds of the whole GPU queued on a few dozen lines.
+// Per-tile pair counters sit one 32-byte sector apart: every pair of the frame
+// adds to one of them, and packed 32 to an L2 line the adds of the whole GPU
+// queued on a few dozen lines.  Word 0 counts the narrow items' pairs (after the
+// scan: the tile's first list place), word 1 the wide items' (after the scan:
+// their emit cursor).
 constexpr int TC_STRIDE = 8;
 
 enum Region {

@@ -29,15 +29,15 @@ bool side_stream(cudaStream_t s, cudaStream_t& side, cudaEvent_t& fork, cudaEven
 cudaError_t launch_project(const Cams& cams, const RParams& P, const float* means, const float* scales, const float* quats,
                            const float* opac, float4* rec, BinRec* binrec, uint32_t* count, uint32_t* tile_cnt,
                            uint32_t* vis_list, uint32_t* wide_list, uint32_t* unb_list, int32_t* splat_slot,
-                           int32_t* slot_surf, Status* st, int num_sms, cudaStream_t stream);
+                           int32_t* slot_surf, uint32_t* pairs, Status* st, int num_sms, cudaStream_t stream);
 cudaError_t set_hold_scan(int hold);  // fss_test_hold_scan
 __global__ void k_emit(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
                        const BinRec* __restrict__ binrec, const uint32_t* __restrict__ vis_list,
                        const uint32_t* __restrict__ wide_list, const uint32_t* __restrict__ unb_list,
                        uint32_t* __restrict__ cursor, int2* __restrict__ ranges, int32_t* __restrict__ order,
-                       uint32_t* __restrict__ list, const float* __restrict__ means, const float* __restrict__ scales,
-                       const float* __restrict__ quats, float4* __restrict__ rec, Status* __restrict__ st,
-                       int max_lines);
+                       uint32_t* __restrict__ list, const uint32_t* __restrict__ pairs, const float* __restrict__ means,
+                       const float* __restrict__ scales, const float* __restrict__ quats, float4* __restrict__ rec,
+                       Status* __restrict__ st, int max_lines);
 __global__ void k_tile_sort(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
                             const BinRec* __restrict__ binrec,
                             const int2* __restrict__ ranges, uint32_t* __restrict__ list,

@@ -303,23 +303,12 @@ __device__ __forceinline__ int warp_line_prefix(const WarpLines& w, int nl) {
     return __shfl_sync(0xffffffffu, incl, 31);
 }
 
-// g(owner lane, item, camera, rows, outer line, first tile, last tile) for
-// every non-empty line interval of the warp's items (inner tiles a..b)
-template <typename G>
-__device__ __forceinline__ void warp_lines(const Cams& cams, const RParams& P, const WarpLines& w, int total, G&& g) {
-    const int lane = threadIdx.x & 31;
-    for (int u = lane; u < total; u += 32) {
-        int j = 0;  // owner: the first lane whose inclusive prefix exceeds u
+// owner lane of unit u: the first lane whose inclusive prefix exceeds u
+__device__ __forceinline__ int unit_owner(const WarpLines& w, int u) {
+    int j = 0;
 #pragma unroll
-        for (int step = 16; step > 0; step >>= 1) j += w.pre[j + step - 1] <= u ? step : 0;
-        const BinRec r = w.br[j];
-        const Lines L = lines_of(r, P.bin_mode);
-        const int o = L.first + (u - (w.pre[j] - L.n));
-        int a, b;
-        if (!line_interval(r, L, P.ts, o, a, b)) continue;
-        const uint32_t item = w.item[j];
-        g(j, item, cams.c[view_of_item(item, P.N)], L.rows, o, a, b);
-    }
+    for (int step = 16; step > 0; step >>= 1) j += w.pre[j + step - 1] <= u ? step : 0;
+    return j;
 }
 
 }  // namespace
@@ -412,11 +401,13 @@ constexpr int PROJ_THREADS = 256;
 // one thread per item, and queues the rest in shared memory; stage B runs the
 // exact culls and the chain one thread per queued item, so the few visible
 // surfels of a view fill whole warps instead of one lane in each.  A visible
-// item with a bounded conic counts its tiles (fire-and-forget adds into the
-// per-tile counters, cleared by the host call before this kernel) and is
-// appended to the narrow list, or to the wide list when it spans more than
-// WIDE_TILES tiles; an unbounded item goes to its view's list instead (every
-// tile of the view includes it).  Appends and gradient-slot claims are
+// item with a bounded conic is appended to the narrow list, or to the wide list
+// when its outer rectangle has more than WIDE_TILES tiles; an unbounded item
+// goes to its view's list instead (every tile of the view includes it).  A
+// narrow item's pairs are made here: each takes the next slot of its tile (the
+// value its add to the tile's counter returns) and goes into a pair buffer as
+// (tile, slot, item), so that k_emit only has to place them once the tiles'
+// first places are known.  A wide item only counts its tiles.  Appends and gradient-slot claims are
 // aggregated per warp.
 //
 // PER = 4 packs stage B well where most items are culled; PER = 1 spreads few
@@ -426,7 +417,12 @@ constexpr int PROJ_THREADS = 256;
 // with the exact culls in it (a logarithm, a square root and four divisions per
 // item) 1.5M items took 50 us where this takes 42, and 12M items 279 / 220.
 // ---------------------------------------------------------------------------
-constexpr uint32_t WIDE_TILES = 32;
+// Wide items: outer rectangles of more tiles than this.  They pay a walk over
+// their lines in k_emit with a warp per line, so only those whose runs would
+// keep one lane busy for long are wide (at 32 the forward of 1.5M surfels at 1280
+// x 720 took 443 us, at 64 417, at 128 408, from 256 on 407).
+constexpr uint32_t WIDE_TILES = 256;
+constexpr int PAIR_BATCH = 8;  // tile counters added to at once by a lane (4: 411 us)
 constexpr int64_t PROJ_SPREAD = 1024;  // items per SM below which a CTA takes 256 of them
 
 template <int PER>
@@ -437,8 +433,8 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
                                                  uint32_t* __restrict__ count, uint32_t* __restrict__ tile_cnt,
                                                  uint32_t* __restrict__ vis_list, uint32_t* __restrict__ wide_list,
                                                  uint32_t* __restrict__ unb_list, int32_t* __restrict__ splat_slot,
-                                                 int32_t* __restrict__ slot_surf, Status* __restrict__ st, float rmax,
-                                                 float mmax) {
+                                                 int32_t* __restrict__ slot_surf, uint32_t* __restrict__ pairs,
+                                                 Status* __restrict__ st, float rmax, float mmax) {
     constexpr int PROJ_ITEMS = PER * PROJ_THREADS;
     __shared__ uint32_t s_q[PROJ_ITEMS];
     __shared__ int s_nq;
@@ -447,8 +443,13 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     __shared__ int s_pre[PROJ_THREADS];
     const int wb = threadIdx.x & ~31;
     const WarpLines wl{s_br + wb, s_item + wb, s_pre + wb};
-    if (st->err) return;
     const int lane = threadIdx.x & 31;
+    const bool one_view = cams.n == 1;  // every item is a surfel of its own: its gradient slot is written here
+    if (st->err) {                      // an error not read yet: nothing but the empty slots
+        for (int k = threadIdx.x; one_view && k < PROJ_ITEMS; k += PROJ_THREADS)
+            if ((int64_t)blockIdx.x * PROJ_ITEMS + k < P.n_items) splat_slot[(int64_t)blockIdx.x * PROJ_ITEMS + k] = -1;
+        return;
+    }
     if (threadIdx.x == 0) s_nq = 0;
     __syncthreads();
     // stage A: the superset of the culls for PROJ_ITEMS items (each thread's items
@@ -470,6 +471,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
         const int k = threadIdx.x + i * PROJ_THREADS;
         const int64_t it = base + k;
         const bool keep = it < P.n_items && !surely_culled(cams.c[vw[i]], P, in[i], rmax, mmax);
+        if (one_view && !keep && it < P.n_items) splat_slot[it] = -1;
         const unsigned m = __ballot_sync(0xffffffffu, keep);
         int b = 0;
         if (lane == 0 && m) b = atomicAdd(&s_nq, __popc(m));
@@ -657,31 +659,85 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
             binrec[item] = br;
             // one gradient slot per surfel visible in any view (-1 -> -2 claims it);
             // with one view every item is a distinct surfel, so no round trip
-            claim = cams.n == 1 || atomicCAS(&splat_slot[s], -1, -2) == -1;
+            claim = one_view || atomicCAS(&splat_slot[s], -1, -2) == -1;
             claim_s = s;
+        } else if (one_view) {
+            splat_slot[s] = -1;
         }
     }
-    // per-tile pair counts (S20 intervals), the warp's lines spread over its lanes
+    // the pairs (S20 intervals), the warp's lines spread over its lanes
+    wide = vis && (br.tx1 - br.tx0 + 1) * (br.ty1 - br.ty0 + 1) > (int)WIDE_TILES;
     {
         const int lane = threadIdx.x & 31;
         if (vis) wl.br[lane] = br;
         wl.item[lane] = (uint32_t)item;
         s_cnt[threadIdx.x] = 0u;
+        const unsigned wides = __ballot_sync(0xffffffffu, wide);
         const int total = warp_line_prefix(wl, vis ? lines_of(br, P.bin_mode).n : 0);
-        warp_lines(cams, P, wl, total, [&](int j, uint32_t, const CamDev& cam, bool rows, int o, int a, int b) {
-            for (int k = a; k <= b; ++k) {
-                const int tx = rows ? k : o, ty = rows ? o : k;
-                const int tt = cam.tile_off + ty * cam.tiles_x + tx;
-                if (in_bounds(st, SITE_TILE, tt, cams.total_tiles)) atomicAdd(&tile_cnt[(size_t)tt * TC_STRIDE], 1u);
+        for (int u0 = 0; u0 < total; u0 += 32) {  // warp-uniform
+            const int u = u0 + lane;
+            int j = 0, len = 0, t0 = 0, step = 1;  // the run of tiles t0 + i * step of one line
+            if (u < total) {
+                j = unit_owner(wl, u);
+                const BinRec r = wl.br[j];
+                const Lines L = lines_of(r, P.bin_mode);
+                const int o = L.first + (u - (wl.pre[j] - L.n));
+                int a, b;
+                if (line_interval(r, L, P.ts, o, a, b)) {
+                    const CamDev& cam = cams.c[view_of_item(wl.item[j], P.N)];
+                    len = b - a + 1;
+                    t0 = cam.tile_off + (L.rows ? o * cam.tiles_x + a : a * cam.tiles_x + o);
+                    step = L.rows ? 1 : cam.tiles_x;
+                    atomicAdd(&s_cnt[wb + j], (uint32_t)len);
+                }
             }
-            atomicAdd(&s_cnt[wb + j], (uint32_t)(b - a + 1));
-        });
-        __syncwarp();
-        if (vis) {
-            const uint32_t cnt = s_cnt[threadIdx.x];
-            count[item] = cnt;
-            wide = cnt > WIDE_TILES;
+            const bool many = (wides >> j) & 1u;
+            // places of the narrow runs in the pair buffer (one atomic per 32 lines)
+            const int mine = many ? 0 : len;
+            int incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            uint32_t at = 0u;
+            if (lane == 31 && incl) at = atomicAdd(&st->npair, (uint32_t)incl);
+            if (many) {
+                for (int i = 0; i < len; ++i)
+                    if (in_bounds(st, SITE_TILE, t0 + i * step, cams.total_tiles))
+                        atomicAdd(&tile_cnt[(size_t)(t0 + i * step) * TC_STRIDE + 1], 1u);
+            }
+            // each pair takes the next slot of its tile; PAIR_BATCH adds in flight
+            uint32_t slot[PAIR_BATCH];
+#pragma unroll
+            for (int i = 0; i < PAIR_BATCH; ++i)
+                slot[i] = i < mine && in_bounds(st, SITE_TILE, t0 + i * step, cams.total_tiles)
+                              ? atomicAdd(&tile_cnt[(size_t)(t0 + i * step) * TC_STRIDE], 1u) : 0u;
+            at = __shfl_sync(0xffffffffu, at, 31) + (uint32_t)(incl - mine);
+            const uint32_t cap = (uint32_t)P.pair_cap, it = wl.item[j];
+            uint32_t* const p_tile = pairs;
+            uint32_t* const p_slot = pairs + cap;
+            uint32_t* const p_item = pairs + 2 * (size_t)cap;
+            for (int i0 = 0; i0 < mine; i0 += PAIR_BATCH) {
+                if (i0 > 0) {
+#pragma unroll
+                    for (int i = 0; i < PAIR_BATCH; ++i)
+                        slot[i] = i0 + i < mine && in_bounds(st, SITE_TILE, t0 + (i0 + i) * step, cams.total_tiles)
+                                      ? atomicAdd(&tile_cnt[(size_t)(t0 + (i0 + i) * step) * TC_STRIDE], 1u) : 0u;
+                }
+#pragma unroll
+                for (int i = 0; i < PAIR_BATCH; ++i) {
+                    const uint32_t q = at + (uint32_t)(i0 + i);
+                    if (i0 + i < mine && q < cap) {  // (over capacity: counted, the frame is reported)
+                        p_tile[q] = (uint32_t)(t0 + (i0 + i) * step);
+                        p_slot[q] = slot[i];
+                        p_item[q] = it;
+                    }
+                }
+            }
         }
+        __syncwarp();
+        if (vis) count[item] = s_cnt[threadIdx.x];
         __syncwarp();  // the slices are reused by the warp's next survivors
     }
     // warp-aggregated appends (one global atomic per warp and counter, no CTA barrier)
@@ -722,7 +778,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
 cudaError_t launch_project(const Cams& cams, const RParams& P, const float* means, const float* scales, const float* quats,
                            const float* opac, float4* rec, BinRec* binrec, uint32_t* count, uint32_t* tile_cnt,
                            uint32_t* vis_list, uint32_t* wide_list, uint32_t* unb_list, int32_t* splat_slot,
-                           int32_t* slot_surf, Status* st, int num_sms, cudaStream_t stream) {
+                           int32_t* slot_surf, uint32_t* pairs, Status* st, int num_sms, cudaStream_t stream) {
     // the largest binning radius per unit scale and screen margin of an opacity <= 1, widened (see surely_culled)
     const double k2 = 2.0 * std::log(1.0 / (double)P.alpha_min) * 1.0009765625;
     const float rmax = (float)(std::sqrt(std::max(k2, 0.0)) * 1.0015);
@@ -732,7 +788,7 @@ cudaError_t launch_project(const Cams& cams, const RParams& P, const float* mean
         const int64_t blocks = std::max<int64_t>(1, (P.n_items + PER * PROJ_THREADS - 1) / (PER * PROJ_THREADS));
         k_project<PER><<<(unsigned)blocks, PROJ_THREADS, 0, stream>>>(cams, P, means, scales, quats, opac, rec, binrec,
                                                                     count, tile_cnt, vis_list, wide_list, unb_list,
-                                                                    splat_slot, slot_surf, st, rmax, mmax);
+                                                                    splat_slot, slot_surf, pairs, st, rmax, mmax);
         return cudaGetLastError();
     };
     return P.n_items < PROJ_SPREAD * num_sms ? go(std::integral_constant<int, 1>{}) : go(std::integral_constant<int, 4>{});
@@ -761,12 +817,15 @@ __device__ void scan_tiles(const Cams& cams, const RParams& P, uint32_t* __restr
     const int nt = cams.total_tiles;
     constexpr int ITEMS = 8;
     for (int base = 0; base < nt; base += blockDim.x * ITEMS) {
-        uint32_t v[ITEMS];
+        uint32_t v[ITEMS], narrow[ITEMS];
         uint32_t sum = 0;
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
             const int t = base + threadIdx.x * ITEMS + k;
-            v[k] = t < nt ? tile_cnt[(size_t)t * TC_STRIDE] + st->unb_cnt[view_of_tile(cams, t)] : 0u;
+            // (both words of the sector at once)
+            const uint2 c = t < nt ? *reinterpret_cast<const uint2*>(tile_cnt + (size_t)t * TC_STRIDE) : make_uint2(0u, 0u);
+            narrow[k] = c.x;
+            v[k] = t < nt ? c.x + c.y + st->unb_cnt[view_of_tile(cams, t)] : 0u;
             sum += v[k];
         }
         uint32_t incl = sum;
@@ -796,7 +855,9 @@ __device__ void scan_tiles(const Cams& cams, const RParams& P, uint32_t* __restr
                 run += v[k];
                 const bool fits = run <= (uint64_t)P.pair_cap;
                 ranges[t] = make_int2(fits ? (int)s0 : 0, fits ? (int)run : 0);
-                tile_cnt[(size_t)t * TC_STRIDE] = fits ? (uint32_t)s0 : 0u;  // emit cursor
+                // first place of the narrow pairs, cursor of the wide ones
+                *reinterpret_cast<uint2*>(tile_cnt + (size_t)t * TC_STRIDE) =
+                    fits ? make_uint2((uint32_t)s0, (uint32_t)s0 + narrow[k]) : make_uint2(0u, 0u);
             }
         }
         __syncthreads();
@@ -942,21 +1003,6 @@ __device__ __forceinline__ void record_item(const Cams& cams, const RParams& P, 
     rr[3].w = ldexp32(fm(n2.hi, n2.hi), -ex);  // total scale of M relative to adj(T' of the normalised surfel)
 }
 
-constexpr int EMIT_BATCH = 8;
-
-// one slot in each of tiles tb[0, n) for `item`: all cursor atomics first, then the stores
-__device__ __forceinline__ void emit_batch(uint32_t* __restrict__ cursor, uint32_t* __restrict__ list,
-                                           const uint32_t* tb, int n, uint32_t item, int64_t cap, int ntiles,
-                                           Status* st) {
-    uint32_t pos[EMIT_BATCH];
-#pragma unroll
-    for (int j = 0; j < EMIT_BATCH; ++j)
-        if (j < n) pos[j] = in_bounds(st, SITE_TILE, tb[j], ntiles) ? atomicAdd(&cursor[(size_t)tb[j] * TC_STRIDE], 1u) : ~0u;
-#pragma unroll
-    for (int j = 0; j < EMIT_BATCH; ++j)
-        if (j < n && pos[j] < (uint32_t)cap) list[pos[j]] = item;
-}
-
 // ---------------------------------------------------------------------------
 // k_emit: writes every bounded visible item into one slot of each of its
 // tiles (slot order is arbitrary; the per-tile sort restores a total order)
@@ -967,8 +1013,11 @@ __device__ __forceinline__ void emit_batch(uint32_t* __restrict__ cursor, uint32
 //                 wait for the flag ends however the CTAs are scheduled;
 //   records:      one thread per narrow, wide or unbounded item (they need no
 //                 ranges, so they run while the scan does);
-//   narrow items: 32 per warp, their (item, outer line) units spread over
-//                 the lanes; each lane emits its line's tiles;
+//   narrow pairs: one thread per (tile, slot, item) that k_project made: the
+//                 item goes to the slot's place in the tile's range (a second
+//                 walk over the lines with one more add per pair took
+//                 24 us for 500k surfels at 640 x 480 where this and the pair's
+//                 making take 19);
 //   wide items:   one warp per (item, outer line), lanes over the line's tiles;
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
@@ -976,12 +1025,10 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Cams cams,
                                               const uint32_t* __restrict__ wide_list,
                                               const uint32_t* __restrict__ unb_list, uint32_t* __restrict__ cursor,
                                               int2* __restrict__ ranges, int32_t* __restrict__ order,
-                                              uint32_t* __restrict__ list, const float* __restrict__ means,
-                                              const float* __restrict__ scales, const float* __restrict__ quats,
-                                              float4* __restrict__ rec, Status* __restrict__ st, int max_lines) {
-    __shared__ BinRec s_br[256];
-    __shared__ uint32_t s_item[256];
-    __shared__ int s_pre[256];
+                                              uint32_t* __restrict__ list, const uint32_t* __restrict__ pairs,
+                                              const float* __restrict__ means, const float* __restrict__ scales,
+                                              const float* __restrict__ quats, float4* __restrict__ rec,
+                                              Status* __restrict__ st, int max_lines) {
     __shared__ int s_scanner, s_go;
     if (st->err) return;
     Status* const stw = st;
@@ -995,8 +1042,6 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Cams cams,
         heavy_first_order(cams, ranges, order);
     }
     const int lane = threadIdx.x & 31;
-    const int wb = threadIdx.x & ~31;
-    const WarpLines wl{s_br + wb, s_item + wb, s_pre + wb};
     const uint32_t nvis = st->nvis, nwide = st->nwide;
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
@@ -1033,38 +1078,15 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Cams cams,
     }
     __syncthreads();
     if (!s_go) return;
-    // narrow items, 32 per warp from the highest warps down (so that they run
-    // beside the records); each lane emits one line's tiles in batches of
-    // EMIT_BATCH, whose cursor atomics are in flight together
-    const int64_t warps = gstride >> 5;
-    for (int64_t c0 = (warps - 1 - (gtid >> 5)) * 32; c0 < nvis; c0 += warps * 32) {  // warp-uniform
-        const int64_t i = c0 + lane;
-        bool ok = i < nvis && in_bounds(stw, SITE_VIS_LIST, i, P.n_items);
-        const uint32_t item = ok ? vis_list[i] : 0u;
-        ok = ok && in_bounds(stw, SITE_ITEM, item, P.n_items);
-        int nl = 0;
-        if (ok) {
-            const BinRec r = binrec[item];
-            wl.br[lane] = r;
-            nl = lines_of(r, P.bin_mode).n;
-        }
-        wl.item[lane] = item;
-        const int total = warp_line_prefix(wl, nl);
-        warp_lines(cams, P, wl, total, [&](int, uint32_t it, const CamDev& cam, bool rows, int o, int a, int b) {
-            uint32_t tb[EMIT_BATCH];
-            int nb = 0;
-            for (int k = a; k <= b; ++k) {
-                const int tx = rows ? k : o, ty = rows ? o : k;
-                tb[nb++] = (uint32_t)(cam.tile_off + ty * cam.tiles_x + tx);
-                if (nb == EMIT_BATCH) {
-                    emit_batch(cursor, list, tb, nb, it, P.pair_cap, cams.total_tiles, stw);
-                    nb = 0;
-                }
-            }
-            emit_batch(cursor, list, tb, nb, it, P.pair_cap, cams.total_tiles, stw);
-        });
-        __syncwarp();  // the slices are reused by the warp's next chunk
+    // the narrow pairs, each to its slot of its tile's range
+    const int64_t npair = min((int64_t)st->npair, P.pair_cap);
+    for (int64_t i = gstride - 1 - gtid; i < npair; i += gstride) {  // (from the threads without a record up)
+        const uint32_t t = pairs[i], slot = pairs[P.pair_cap + i];
+        if (!in_bounds(stw, SITE_TILE, t, cams.total_tiles)) continue;
+        const uint32_t pos = __ldcg(cursor + (size_t)t * TC_STRIDE) + slot;  // (written during this kernel: from L2)
+        if (pos < (uint32_t)P.pair_cap) list[pos] = pairs[2 * P.pair_cap + i];
     }
+    const int64_t warps = gstride >> 5;
     // wide items: one warp per (item, outer line), lanes over the line's tiles,
     // so that a surfel spanning many tiles is spread over many warps
     const int64_t units = (int64_t)nwide * max_lines;
@@ -1085,7 +1107,7 @@ __global__ void __launch_bounds__(256) k_emit(const __grid_constant__ Cams cams,
             const int tx = L.rows ? k : o, ty = L.rows ? o : k;
             const int tt = cam.tile_off + ty * cam.tiles_x + tx;
             if (!in_bounds(stw, SITE_TILE, tt, cams.total_tiles)) continue;
-            const uint32_t pos = atomicAdd(&cursor[(size_t)tt * TC_STRIDE], 1u);
+            const uint32_t pos = atomicAdd(&cursor[(size_t)tt * TC_STRIDE + 1], 1u);
             if (pos < (uint32_t)P.pair_cap) list[pos] = item;
         }
     }
