@@ -263,7 +263,7 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
     const size_t smem = query_labels_smem(nq, 8 * KC);
     auto kern = k_query_labels<KC>;
     cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) {
+    if (smem + 1024 > 48 * 1024) {  // with the static shared memory
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
@@ -298,11 +298,11 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
 // with FP32 against 31.1 and 36.7; 80 x 48 59.2 and 81.2 against 61.1 and 67.7.
 // FP32 labels store twice the bytes: from 80 queries on query_wide.cu is ahead
 // (112 x 64: 123 / 91 us).  BF16 labels gain less (112 x 64 91.2 / 84.5, 128 x
-// 96 120.5 / 99.2) and lose below 100k Gaussians (50,000 x 112 x 48 14.1 / 16.2)
+// 96 120.5 / 99.2) and lose on fewer Gaussians (100k x 112 x 48 21.1 / 23.8)
 // and above 96 channels, where shared memory leaves query_wide.cu fewer
 // Gaussians per SM (128 x 128 with 1.3M: 292 / 332).
 bool wide_queries(int64_t N, int nq, int dim, bool bf16) {
-    return bf16 ? nq >= 96 && dim <= 96 && N >= 100000 : nq >= 80;
+    return bf16 ? nq >= 96 && dim <= 96 && N >= 200000 : nq >= (N >= 100000 ? 80 : 96);
 }
 
 }  // namespace

@@ -349,13 +349,16 @@ size_t query_smem(int qb, int nbuf, int nq, int dim) {
 template <int QB, typename OT>
 cudaError_t launch_qb(int64_t N, int nq, int dim, int ncols, int nbuf, const void* f_ins, const float* means, const void* f_q,
                       const float* p_q, const float* prec, void* out, int32_t* err, int num_sms, cudaStream_t stream) {
-    const size_t smem = query_smem(QB, nbuf, nq, dim);
+    size_t smem = query_smem(QB, nbuf, nq, dim);
     auto kern = k_query_wide<QB, OT>;
+    // resident CTAs per SM: by the registers (the launch bounds), the SM's
+    // tensor memory (512 columns) and shared memory.  The request is raised until
+    // no more than these fit: a CTA beyond them would wait for tensor memory until
+    // another one has done all its tiles (865k x 144 x 32 in FP32: 306 us, 195.02 without)
+    const int per_sm = std::max(1, std::min({QB == 2 ? 2 : 3, 512 / (QB * ncols), (int)(227 * 1024 / (smem + 4 * 1024))}));
+    smem = std::max(smem, (size_t)(227 * 1024 / (per_sm + 1)));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // resident CTAs per SM: by the registers (the launch bounds), the SM's
-    // tensor memory (512 columns) and shared memory
-    const int per_sm = std::max(1, std::min({QB == 2 ? 2 : 3, 512 / (QB * ncols), (int)(227 * 1024 / (smem + 4 * 1024))}));
     const int64_t ntiles = (N + QM * QB - 1) / (QM * QB);
     const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms);
     kern<<<grid, QTHREADS, smem, stream>>>(N, nq, dim / 8, ncols, nbuf, static_cast<const __nv_bfloat16*>(f_ins), means,
