@@ -260,31 +260,27 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
                       const float* prec, void* out, int out_bf16, int32_t* err, int num_sms, cudaStream_t stream) {
     int ncols = 32;
     while (ncols < nq) ncols <<= 1;
-    size_t smem = query_labels_smem(nq, 8 * KC);
+    const size_t smem = query_labels_smem(nq, 8 * KC);
     auto kern = k_query_labels<KC>;
+    cudaError_t e = cudaSuccess;
+    if (smem + 1024 > 48 * 1024) {  // with the static shared memory
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     // resident CTAs per SM from the kernel's registers and shared memory (the
     // occupancy query answers 1 for this tensor-memory kernel), at most the
-    // number whose tensor-memory columns fit the SM's 512 together; where those
-    // are the limit the shared-memory request is raised so that no more fit (a
-    // CTA beyond them would wait there until another one has done all its tiles)
+    // number whose tensor-memory columns fit the SM's 512 together
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return e;
     int dev = 0, smem_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     if (e != cudaSuccess) return e;
     const int regs = ((std::max(fa.numRegs, 1) + 7) & ~7) * QTHREADS;
-    int per_sm = std::min({2048 / QTHREADS, 65536 / regs, smem_sm / (int)(smem + fa.sharedSizeBytes + 1024)});
-    if (512 / ncols < per_sm) {
-        per_sm = 512 / ncols;
-        smem = std::max(smem, (size_t)(smem_sm / (per_sm + 1)));
-    }
+    int per_sm = std::min({2048 / QTHREADS, 65536 / regs, smem_sm / (int)(smem + fa.sharedSizeBytes + 1024),
+                           512 / ncols});
     per_sm = std::max(1, per_sm);
-    if (smem + 1024 > 48 * 1024) {  // with the static shared memory
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
     const int64_t ntiles = (N + QM - 1) / QM;
     const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms);
     kern<<<grid, QTHREADS, smem, stream>>>(N, nq, ncols, static_cast<const __nv_bfloat16*>(f_ins), means,
@@ -302,11 +298,11 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
 // with FP32 against 31.1 and 36.7; 80 x 48 59.2 and 81.2 against 61.1 and 67.7.
 // FP32 labels store twice the bytes: from 80 queries on query_wide.cu is ahead
 // (112 x 64: 123 / 91 us).  BF16 labels gain less (112 x 64 91.2 / 84.5, 128 x
-// 96 120.5 / 99.2) and lose on fewer Gaussians (200k x 112 x 48 35.8 / 39.5)
+// 96 120.5 / 99.2) and lose on fewer Gaussians (100k x 112 x 48 21.1 / 23.8)
 // and above 96 channels, where shared memory leaves query_wide.cu fewer
 // Gaussians per SM (128 x 128 with 1.3M: 292 / 332).
 bool wide_queries(int64_t N, int nq, int dim, bool bf16) {
-    return bf16 ? nq >= 96 && dim <= 96 && N >= 300000 : nq >= (N >= 100000 ? 80 : 96);
+    return bf16 ? nq >= 96 && dim <= 96 && N >= 200000 : nq >= (N >= 100000 ? 80 : 96);
 }
 
 }  // namespace
