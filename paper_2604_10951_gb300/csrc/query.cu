@@ -297,12 +297,16 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
 // a tile is little work: 500k x 32 x 32 takes 27.1 us with BF16 labels and 38.2
 // with FP32 against 31.1 and 36.7; 80 x 48 59.2 and 81.2 against 61.1 and 67.7.
 // FP32 labels store twice the bytes: from 80 queries on query_wide.cu is ahead
-// (112 x 64: 123 / 91 us).  BF16 labels gain less (112 x 64 91.2 / 84.5, 128 x
-// 96 120.5 / 99.2) and lose on fewer Gaussians (100k x 112 x 48 21.1 / 23.8)
-// and above 96 channels, where shared memory leaves query_wide.cu fewer
-// Gaussians per SM (128 x 128 with 1.3M: 292 / 332).
+// (112 x 64: 123 / 91 us).  BF16 labels gain less: with more than 128 queries
+// or 48 channels (200k x 160 x 16 60.6 / 46.5, 224 x 48 74.9 / 65.8, 96 x 96
+// 41.9 / 38.4; 1.2M x 112 x 64 91.2 / 84.5).  With fewer of both the kernel
+// above is ahead or level (112 x 48 with 200k 35.7 / 38.8, with 500k 77.5 /
+// 79.7), as it is on fewer Gaussians (100k x 112 x 48 21.1 / 23.8) and above 96
+// channels, where shared memory leaves query_wide.cu fewer Gaussians per SM
+// (128 x 128 with 1.3M: 292 / 332).
 bool wide_queries(int64_t N, int nq, int dim, bool bf16) {
-    return bf16 ? nq >= 96 && dim <= 96 && N >= 200000 : nq >= (N >= 100000 ? 80 : 96);
+    if (!bf16) return nq >= (N >= 100000 ? 80 : 96);
+    return N >= 200000 && nq >= 96 && dim <= 96 && (nq > 128 || dim > 48);
 }
 
 }  // namespace

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("n,nq,dim,dtype", [
     (1, 96, 16, torch.float32), (127, 96, 48, torch.float32), (129, 96, 128, torch.float32),
     (255, 112, 64, torch.float32), (257, 176, 112, torch.float32), (1000, 256, 128, torch.float32),
-    (78_001, 112, 32, torch.float32), (78_080, 144, 80, torch.float32), (200_003, 112, 16, torch.bfloat16),
+    (78_001, 112, 32, torch.float32), (78_080, 144, 80, torch.float32), (200_003, 96, 64, torch.bfloat16),
     (200_000, 144, 96, torch.bfloat16)])
 def test_wide_labels_against_oracle(n, nq, dim, dtype):
     means = scenes.room_scene(n=max(n, 5000), C=4, seed=n).means[:n]
