@@ -8,7 +8,7 @@
 //   S_{j-1} = a_j s_j + (1 - a_j) S_j,  T_j = T_{j+1} / (1 - a_j)
 // replayed back to front from the saved traversal length and final T.
 //
-// k_bwd_feat  (Top-K) one CTA per tile: for every selected (pixel, k) the
+// k_bwd_feat  (Top-K, except where k_bwd_geo_topk does it) one CTA per tile: for every selected (pixel, k) the
 //             dot c_i . dL/dF(x) and the feature gradient sum w_i dL/dF(x),
 //             grouped by surfel in shared memory first, so each surfel's
 //             feature row is read once and costs one row of 16-byte vector
@@ -642,12 +642,30 @@ __global__ void __launch_bounds__(TS * TS) k_bwd_geo_full(const __grid_constant_
 // 640 x 480 frame of 500k surfels, 88 here; 1296 x 968 with K = 24 324 / 305.
 // Bound by instruction issue: about 40 of a warp evaluation's instructions are
 // the record, the ray and the derivatives, 55 the reduce-scatter.
+constexpr int FEAT_IN_GEO_C = 32, FEAT_IN_GEO_K = 9;  // see feat_in_geo
 constexpr int GEO_THREADS = 128;  // threads per CTA (64 for 8 x 8 tiles): parts of a tile
 
+// CF > 0 instances (16 or 32: channels, rounded up) also take the feature
+// gradients: the dot c_j . dL/dF from the surfel's staged row and the pixel's
+// gradient in registers, and one more reduce-scatter of w dL/dF per surfel that
+// any of the warp's pixels selected.  The feature kernel, which groups K entries
+// per pixel by surfel in shared memory first, and its dots in memory are then not
+// needed: 1296 x 968, 16 channels, K = 24 FP32 geometry and features 860 us
+// before, 555 here (step 1573 / 1264).  Bound by instruction issue: 16 selects and
+// multiplies and 17 shuffles per surfel and warp for 16 channels.
+template <int CF, typename FT>
 struct GeoStage {
     WarpStage st[2];
     int32_t slot[2][32];
+    FT row[CF ? 2 : 1][CF ? 32 : 1][CF ? CF + 16 / (int)sizeof(FT) : 1];  // feature rows, padded by 16 bytes
 };
+
+// threads per CTA: 64 where the stages of four warps are above 48 KB
+template <int TS, int CF, typename FT>
+constexpr int geo_threads() {
+    const int nt = CF && 4 * sizeof(GeoStage<CF, FT>) > 47 * 1024 ? GEO_THREADS / 2 : GEO_THREADS;
+    return TS * TS < nt ? TS * TS : nt;
+}
 
 // warp sums of v[0..12]: afterwards an even lane l < 26 holds the sum of v[l >> 1]
 __device__ __forceinline__ void reduce_scatter13(float (&v)[13]) {
@@ -675,17 +693,25 @@ __device__ __forceinline__ void reduce_scatter13(float (&v)[13]) {
     v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-template <int TS, bool VAR>
-__global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
-                                  1024 / (TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS))
+template <int TS, bool VAR, int CF = 0, typename FT = float>
+__global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
+                                  (CF == 0 ? 1024 : CF == 16 ? 768 : 512) / geo_threads<TS, CF, FT>())
     k_bwd_geo_topk(const __grid_constant__ Cams cams, const __grid_constant__ RParams P, const BwdArgs a) {
-    constexpr int NT = TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS, NW = NT / 32, PARTS = TS * TS / NT;
+    constexpr int NT = geo_threads<TS, CF, FT>(), NW = NT / 32, PARTS = TS * TS / NT;
     constexpr unsigned ALL = 0xffffffffu;
-    __shared__ __align__(16) GeoStage s_stage[NW];
+    static_assert(!VAR || CF == 0, "the variants take the feature gradients from their own kernel");
+    __shared__ __align__(16) GeoStage<CF, FT> s_stage[NW];
     __shared__ int s_work;
     if (a.st->err) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    GeoStage& G = s_stage[warp];
+    GeoStage<CF, FT>& G = s_stage[warp];
+    constexpr int E = FeatVec<FT>::E;
+    const FT* __restrict__ feats = reinterpret_cast<const FT*>(a.feats);
+    if constexpr (CF > 0) {  // channels past C: zeros, once
+        for (int i = lane; i < 2 * 32 * CF; i += 32)
+            if (i % CF >= P.C) G.row[i / (32 * CF)][(i / CF) % 32][i % CF] = FT(0.0f);
+        __syncwarp();
+    }
     const int K = P.K, total = cams.total_tiles * PARTS;
     for (bool first = true;; first = false) {
         int u;  // this CTA's next part of a tile (heavy tiles first)
@@ -721,7 +747,7 @@ __global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
         int nstop = 0;
         float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
         int kk = -1, next_pos = -1;
-        float next_dot = 0.0f;
+        float next_dot = 0.0f;  // (CF: that surfel's weight)
         // a selected surfel adds rn_a * dot + rn_b to what its weight multiplies:
         // the dot itself, or (dot - F.dL/dF) / W for the renormalised variant
         float rn_a = 1.0f, rn_b = 0.0f;
@@ -736,7 +762,7 @@ __global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
                 if (a.saved_pos[pix * K + kk] >= 0) break;
             if (kk >= 0) {
                 next_pos = a.saved_pos[pix * K + kk];
-                next_dot = a.dots[pix * K + kk];
+                next_dot = (CF == 0 ? a.dots : a.saved_w)[pix * K + kk];
             }
             if (VAR && P.renorm) {  // entries 0..kk are the selected ones, front to back
                 float ws = 0.0f, wd = 0.0f;
@@ -749,12 +775,31 @@ __global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
                 rn_b = -wd * rn_a * rn_a;
             }
         }
+        float2 dfr[CF ? CF / 2 : 1];  // this pixel's dL/dF
+        if constexpr (CF > 0) {
+#pragma unroll
+            for (int v = 0; v < CF / E; ++v) {
+                float f[E];
+#pragma unroll
+                for (int e = 0; e < E; ++e) f[e] = 0.0f;
+                if (inside && v * E < P.C) FeatVec<FT>::load(reinterpret_cast<const FT*>(a.d_feat) + pix * P.C + v * E, f);
+#pragma unroll
+                for (int e = 0; e < E / 2; ++e) dfr[v * (E / 2) + e] = make_float2(f[2 * e], f[2 * e + 1]);
+            }
+        }
         const int L = __reduce_max_sync(ALL, nstop);
 
         // one chunk's records and gradient slots, and the lane mask of those the warp meets
         auto stage = [&](int buf, const ListEntry& e) {
             const int64_t sp = (int64_t)e.item - vbase;
-            if ((e.mask & wbit) && FSS_CHECKED(sp >= 0 && sp < P.N)) cp_async4(&G.slot[buf][lane], a.splat_slot + sp);
+            if ((e.mask & wbit) && FSS_CHECKED(sp >= 0 && sp < P.N)) {
+                cp_async4(&G.slot[buf][lane], a.splat_slot + sp);
+                if constexpr (CF > 0) {
+#pragma unroll
+                    for (int v = 0; v < CF / E; ++v)
+                        if (v * E < P.C) cp_async16(&G.row[buf][lane][v * E], feats + sp * P.C + v * E, 16);
+                }
+            }
             return stage_chunk(G.st[buf], e, wbit, a.rec, rgbv, vbase, P.N, a.st);
         };
         // chunk b0 is worked on while the one before it is copied and the list entries of the next are read
@@ -775,6 +820,8 @@ __global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
 #pragma unroll
                 for (int k = 0; k < (VAR ? 16 : 13); ++k) g[k] = 0.0f;
                 bool contrib = false;
+                bool sel = false;  // CF: this pixel selected the surfel, with the forward's weight
+                float wsel = 0.0f;
                 Hit h;
                 const float4 oc = S.oc[j];
                 if (pos < nstop &&
@@ -785,10 +832,27 @@ __global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
                     const float w = alpha * Tj;
                     float s = oc.y * gr + oc.z * gg + oc.w * gb;
                     if (pos == next_pos) {
-                        s += VAR ? fmaf(next_dot, rn_a, rn_b) : next_dot;
+                        if constexpr (CF > 0) {
+                            float2 d0 = make_float2(0.0f, 0.0f), d1 = d0;
+#pragma unroll
+                            for (int v = 0; v < CF / E; ++v) {
+                                float f[E];
+                                FeatVec<FT>::lds(&G.row[buf][j][v * E], f);
+#pragma unroll
+                                for (int e = 0; e < E / 2; e += 2) {
+                                    d0 = __ffma2_rn(make_float2(f[2 * e], f[2 * e + 1]), dfr[v * (E / 2) + e], d0);
+                                    d1 = __ffma2_rn(make_float2(f[2 * e + 2], f[2 * e + 3]), dfr[v * (E / 2) + e + 1], d1);
+                                }
+                            }
+                            s += (d0.x + d0.y) + (d1.x + d1.y);
+                            sel = true;
+                            wsel = next_dot;
+                        } else {
+                            s += VAR ? fmaf(next_dot, rn_a, rn_b) : next_dot;
+                        }
                         --kk;
                         next_pos = kk >= 0 ? a.saved_pos[pix * K + kk] : -1;
-                        next_dot = kk >= 0 ? a.dots[pix * K + kk] : 0.0f;
+                        next_dot = kk >= 0 ? (CF == 0 ? a.dots : a.saved_w)[pix * K + kk] : 0.0f;
                     }
                     const float dal = Tj * (s - Sh);
                     Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
@@ -817,6 +881,20 @@ __global__ void __launch_bounds__(TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS,
                     const int slot = G.slot[buf][j];
                     if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13) && in_bounds(a.st, SITE_SLOT, slot, P.N))
                         atomicAdd(grows + (int64_t)slot * GRAD_STRIDE + (lane >> 1), g[0]);
+                    if constexpr (CF > 0) {
+                        if (__any_sync(ALL, sel)) {
+                            float gf[CF];
+#pragma unroll
+                            for (int c = 0; c < CF / 2; ++c) {
+                                gf[2 * c] = sel ? wsel * dfr[c].x : 0.0f;  // (dL/dF may be infinite where not selected)
+                                gf[2 * c + 1] = sel ? wsel * dfr[c].y : 0.0f;
+                            }
+                            reduce_scatter<CF>(gf);  // lane l holds channel l (CF = 32) or l >> 1
+                            const int c = CF == 32 ? lane : lane >> 1;
+                            if ((CF == 32 || (lane & 1) == 0) && c < P.C && in_bounds(a.st, SITE_SLOT, slot, P.N))
+                                atomicAdd(a.feat_acc + (int64_t)slot * P.C + c, gf[0]);
+                        }
+                    }
                 }
             }
             word = next;
@@ -1137,30 +1215,45 @@ cudaError_t launch_geo_full(const Cams& cams, const RParams& P, const BwdArgs& a
     return e;
 }
 
-template <int TS>
+// The feature gradients in the replay kernel: the feature kernel's work grows
+// with K, the replay's little.  640 x 480 steps, feature kernel / replay: 16
+// channels FP32 K = 8 196 / 187 us (but the feature rows then no longer run
+// beside the replay when launched eagerly: level), K = 9 242 / 222, K = 32 401 /
+// 300; 32 channels FP32 K = 8 224 / 230, K = 9 278 / 269, K = 32 455 / 380, BF16
+// K = 8 207 / 215, K = 9 254 / 247; 24 channels, 1296 x 968, tiles of 8, 16, 32, K = 16 1.04
+// to 1.17x.  Not with a renormalised selection, which needs every dot before the
+// first, nor with the other variants.
+bool feat_in_geo(const RParams& P) {
+    return P.K >= FEAT_IN_GEO_K && P.C <= FEAT_IN_GEO_C && !P.renorm && !P.color_sh && !P.lowpass;
+}
+
+template <int TS, typename FT>
 cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
-    constexpr int NT = TS * TS < GEO_THREADS ? TS * TS : GEO_THREADS, PARTS = TS * TS / NT;
-    auto go = [&](auto kern) {
-        int64_t units = (int64_t)cams.total_tiles * PARTS;
+    auto go = [&](auto kern, int nt) {
+        int64_t units = (int64_t)cams.total_tiles * (TS * TS / nt);
         if (a.persistent) {
             int wave = (int)std::min<int64_t>(units, INT_MAX);
-            const cudaError_t e = persistent_grid((const void*)kern, NT, 0, wave);
+            const cudaError_t e = persistent_grid((const void*)kern, nt, 0, wave);
             if (e != cudaSuccess) return e;
             units = wave;
         }
-        kern<<<(unsigned)units, NT, 0, s>>>(cams, P, a);
+        kern<<<(unsigned)units, nt, 0, s>>>(cams, P, a);
         const cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) kernel_mark(s);
         return e;
     };
-    return P.renorm || P.color_sh || P.lowpass ? go(k_bwd_geo_topk<TS, true>) : go(k_bwd_geo_topk<TS, false>);
+    if (feat_in_geo(P))
+        return P.C <= 16 ? go(k_bwd_geo_topk<TS, false, 16, FT>, geo_threads<TS, 16, FT>())
+                         : go(k_bwd_geo_topk<TS, false, 32, FT>, geo_threads<TS, 32, FT>());
+    return P.renorm || P.color_sh || P.lowpass ? go(k_bwd_geo_topk<TS, true>, geo_threads<TS, 0, float>())
+                                               : go(k_bwd_geo_topk<TS, false>, geo_threads<TS, 0, float>());
 }
 
 template <int TS, typename FT>
 cudaError_t launch_geo(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
     // the variants (renormalised Top-K, spherical-harmonic colours, low-pass
     // filter) have their own instances: no cost on the plain paths
-    if (P.K > 0) return launch_geo_topk<TS>(cams, P, a, s);
+    if (P.K > 0) return launch_geo_topk<TS, FT>(cams, P, a, s);
     const bool var = P.color_sh || P.lowpass;
     if (P.C <= 32) return var ? launch_geo_full<TS, 32, FT, true>(cams, P, a, s) : launch_geo_full<TS, 32, FT, false>(cams, P, a, s);
     if (P.C <= 64) return var ? launch_geo_full<TS, 64, FT, true>(cams, P, a, s) : launch_geo_full<TS, 64, FT, false>(cams, P, a, s);
@@ -1174,7 +1267,9 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     k_bwd_clear<<<num_sms * 4, 256, 0, s>>>(cams, P, a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     kernel_mark(s);
-    if (P.K > 0) {
+    if (feat_in_geo(P)) {
+        kernel_mark(s);  // the feature gradients' place among the events: nothing runs there
+    } else if (P.K > 0) {
         if ((e = launch_feat<FT>(cams, P, a, s)) != cudaSuccess) return e;
     }
     // With Top-K the feature gradients are complete here: launched eagerly,
@@ -1186,7 +1281,7 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return e;
-    const bool fork = a.g_feat && P.K > 0 && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
+    const bool fork = a.g_feat && P.K > 0 && !feat_in_geo(P) && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
                       side_stream(s, side, ev_fork, ev_join);
     if (fork) {
         if ((e = cudaEventRecord(ev_fork, s)) != cudaSuccess) return e;
