@@ -17,9 +17,8 @@
 //             surfel the warp reduce-scatters its 13 partial derivatives
 //             (adjugate rows 9, opacity 1, colour 3) and adds them to the
 //             surfel's gradient row.
-// k_bwd_geo_full (K = 0) the same with a CTA per tile: it also forms c_j . dL/dF
-//             inline and reduce-scatters the feature gradient, and flushes one
-//             row of vector reductions per surfel and tile.
+// k_bwd_geo_full (K = 0) the same, with c_j . dL/dF and the feature gradients of
+//             every contributor as products shared by the warp's lanes.
 // k_bwd_project one thread per surfel: adjugate-row gradients -> homography
 //             columns -> means, scales, quaternions; sums the views.
 // k_feat_out  writes every row of the feature gradient (zeros for surfels
@@ -28,6 +27,7 @@
 #include "fss_internal.cuh"
 #include "kernels.cuh"
 #include "render_common.cuh"
+#include "render_full.cuh"
 
 #include <algorithm>
 #include <climits>
@@ -411,225 +411,6 @@ __global__ void __launch_bounds__(BWD_FEAT_THREADS, 4) k_bwd_feat(const __grid_c
 }
 
 // ---------------------------------------------------------------------------
-// k_bwd_geo_full: back-to-front replay of the full accumulation (K = 0)
-// ---------------------------------------------------------------------------
-template <int TS, int CMAX, typename FT, bool VAR>
-__global__ void __launch_bounds__(TS * TS) k_bwd_geo_full(const __grid_constant__ Cams cams,
-                                                     const __grid_constant__ RParams P, const BwdArgs a) {
-    constexpr int NT = TS * TS;
-    constexpr int NB = FBATCH;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float4* s_r0 = reinterpret_cast<float4*>(smem);
-    float4* s_r1 = s_r0 + NB;
-    float4* s_r2 = s_r1 + NB;
-    float4* s_oc = s_r2 + NB;                                  // (o, r, g, b)
-    uint32_t* s_wm = reinterpret_cast<uint32_t*>(s_oc + NB);   // warps the footprint reaches
-    float* s_g = reinterpret_cast<float*>(s_wm + 2 * NB);      // [NB][16] partial derivatives
-    float* s_f = s_g + NB * 16;    // [NB][C] features
-    float* s_gf = s_f + NB * P.C;  // [NB][C] feature gradients
-    __shared__ int s_max;
-    __shared__ int s_tile;
-    __shared__ uint32_t s_bits[NT / 32][NB / 32];  // per warp: the staged surfels its block meets
-
-    if (a.st->err) return;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const uint32_t wbit = 1u << (tid >> 5);
-    const int C = P.C;
-    for (int t = next_tile_q(a.persistent, &a.st->work_geo, &s_tile, true, cams); t < cams.total_tiles;
-         t = next_tile_q(a.persistent, &a.st->work_geo, &s_tile, false, cams)) {
-    const int view = view_of_tile(cams, t);
-    const CamDev& cam = cams.c[view];
-    const int lt = t - cam.tile_off;
-    const int tx = lt % cam.tiles_x, ty = lt / cam.tiles_x;
-    const int2 lp = pixel_of<TS>(tid);
-    const int px = tx * TS + lp.x, py = ty * TS + lp.y;
-    const bool inside = px < cam.W && py < cam.H;
-    const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
-    const int2 rg = checked_range(a.ranges, t, P.pair_cap, a.st);
-    const int64_t vbase = (int64_t)view * P.N;
-    // VAR instances carry the variants (spherical-harmonic item colours, low-pass
-    // filter), read from the parameters; the plain instance keeps its code as it is
-    const float* __restrict__ rgbv = a.rgb + (VAR && P.color_sh ? 3 * vbase : 0);
-    const int64_t pix = cam.pix_off + (int64_t)py * cam.W + px;
-    const FT* __restrict__ feats = reinterpret_cast<const FT*>(a.feats);
-
-    int nstop = 0;
-    float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
-    float dfr[CMAX];
-#pragma unroll
-    for (int c = 0; c < CMAX; ++c) dfr[c] = 0.0f;
-    if (inside) {
-        nstop = a.saved_nstop[pix];
-        T = a.out_T[pix];
-        gr = a.d_rgb[3 * pix];
-        gg = a.d_rgb[3 * pix + 1];
-        gb = a.d_rgb[3 * pix + 2];
-        Sh = P.bg[0] * gr + P.bg[1] * gg + P.bg[2] * gb + (a.d_T ? a.d_T[pix] : 0.0f);
-        const FT* dF = reinterpret_cast<const FT*>(a.d_feat) + pix * C;
-#pragma unroll
-        for (int c = 0; c < CMAX; ++c) dfr[c] = c < C ? FeatVec<FT>::one(dF + c) : 0.0f;
-    }
-    if (tid == 0) s_max = 0;
-    __syncthreads();
-    atomicMax(&s_max, nstop);
-    __syncthreads();
-    const int L = s_max;
-
-    for (int b_end = L; b_end > 0; b_end -= NB) {
-        const int b_start = max(0, b_end - NB);
-        const int cnt = b_end - b_start;
-        __syncthreads();
-        for (int j = tid; j < cnt; j += NT) {
-            const uint32_t item = a.list[rg.x + b_start + j];
-            if (!in_bounds(a.st, SITE_ITEM, (int64_t)item - vbase, P.N)) {  // check build: a dead record
-                s_oc[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                s_wm[j] = 0u;
-                continue;
-            }
-            const float4* r = a.rec + 4 * (size_t)item;
-            s_r0[j] = r[0];
-            s_r1[j] = r[1];
-            s_r2[j] = r[2];
-            const int64_t sp = (int64_t)item - vbase;
-            s_oc[j] = make_float4(r[3].x, rgbv[3 * sp], rgbv[3 * sp + 1], rgbv[3 * sp + 2]);
-            s_wm[j] = a.masks[rg.x + b_start + j];
-        }
-        for (int i = tid; i < cnt * 16; i += NT) s_g[i] = 0.0f;
-        {
-            constexpr int E = FeatVec<FT>::E;
-            const int nvec = C / E, rpi = NT / nvec, r0 = tid / nvec, vv = tid - r0 * nvec;
-            for (int j = r0; r0 < rpi && j < cnt; j += rpi) {
-                const int64_t sp = (int64_t)a.list[rg.x + b_start + j] - vbase;
-                if (!FSS_CHECKED(sp >= 0 && sp < P.N)) continue;  // recorded by the staging loop
-                float f[E];
-                FeatVec<FT>::load(feats + sp * C + vv * E, f);
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    s_f[j * C + vv * E + e] = f[e];
-                    s_gf[j * C + vv * E + e] = 0.0f;
-                }
-            }
-        }
-        __syncthreads();
-        // this warp's staged surfels as bit words (the footprint misses the
-        // other ones): the loop below visits set bits only, last first
-#pragma unroll
-        for (int i = 0; i < NB / 32; ++i) {
-            const int j = 32 * i + lane;
-            const uint32_t word = __ballot_sync(0xffffffffu, j < cnt && (s_wm[j] & wbit));
-            if (lane == i) s_bits[tid >> 5][i] = word;
-        }
-        __syncwarp();
-        for (int i = ((cnt + 31) >> 5) - 1; i >= 0; --i) {
-        for (uint32_t bits = s_bits[tid >> 5][i]; bits != 0u; bits ^= 0x80000000u >> __clz(bits)) {
-            const int j = 32 * i + 31 - __clz(bits);
-            const int pos = b_start + j;
-            float g[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) g[k] = 0.0f;
-            float w = 0.0f;
-            bool contrib = false;
-            Hit h;
-            const float4 oc = s_oc[j];
-            if (pos < nstop &&
-                eval_splat<VAR>(s_r0[j], s_r1[j], s_r2[j], oc.x, pxf, pyf, P.alpha_min, cam.near_plane, h, P.lowpass)) {
-                contrib = true;
-                const float alpha = fminf(h.alpha_raw, P.alpha_max);
-                const float Tj = T * rcp_approx(1.0f - alpha);
-                w = alpha * Tj;
-                float s = oc.y * gr + oc.z * gg + oc.w * gb;
-                const float4* fr = reinterpret_cast<const float4*>(s_f + j * C);
-                float d0 = 0.0f, d1 = 0.0f;
-#pragma unroll
-                for (int c4 = 0; c4 < CMAX / 4; ++c4) {
-                    if (4 * c4 < C) {
-                        const float4 fv = fr[c4];
-                        d0 = fmaf(fv.x, dfr[4 * c4], d0);
-                        d1 = fmaf(fv.y, dfr[4 * c4 + 1], d1);
-                        d0 = fmaf(fv.z, dfr[4 * c4 + 2], d0);
-                        d1 = fmaf(fv.w, dfr[4 * c4 + 3], d1);
-                    }
-                }
-                s += d0 + d1;
-                const float dal = Tj * (s - Sh);
-                Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
-                g[10] = w * gr;
-                g[11] = w * gg;
-                g[12] = w * gb;
-                if (h.alpha_raw < P.alpha_max) {
-                    g[9] = dal * h.G;
-                    const float drho = -0.5f * alpha * dal;
-                    if (VAR && h.scr) {  // low-pass screen term: rho = 2 |x - c|^2, d rho / d c = -4 (X, Y)
-                        g[13] = -4.0f * h.X * drho;
-                        g[14] = -4.0f * h.Y * drho;
-                    } else {
-                        const float du = 2.0f * h.u * drho, dv = 2.0f * h.v * drho;
-                        const float gc0 = du * h.inv, gc1 = dv * h.inv, gc2 = -(du * h.u + dv * h.v) * h.inv;
-                        g[0] = gc0 * h.X; g[1] = gc0 * h.Y; g[2] = gc0;
-                        g[3] = gc1 * h.X; g[4] = gc1 * h.Y; g[5] = gc1;
-                        g[6] = gc2 * h.X; g[7] = gc2 * h.Y; g[8] = gc2;
-                    }
-                }
-                T = Tj;
-            }
-            if (__any_sync(0xffffffffu, contrib)) {
-                reduce_scatter<16>(g);  // lane l holds value l >> 1
-                if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13)) atomicAdd(&s_g[j * 16 + (lane >> 1)], g[0]);
-                {
-#pragma unroll
-                    for (int c0 = 0; c0 < CMAX; c0 += 32) {
-                        if (c0 < C) {
-                            float gf[32];
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) gf[c] = w * dfr[c0 + c];
-                            reduce_scatter<32>(gf);  // lane l holds channel c0 + l
-                            if (c0 + lane < C) atomicAdd(&s_gf[j * C + c0 + lane], gf[0]);
-                        }
-                    }
-                }
-            }
-        }
-        }
-        __syncthreads();
-        // flush one gradient row per staged surfel
-        for (int j = tid; j < cnt; j += NT) {
-            const float* v = s_g + 16 * j;
-            bool nz = false;
-#pragma unroll
-            for (int k = 0; k < (VAR ? 15 : 13); ++k) nz |= v[k] != 0.0f;
-            if (!nz) continue;
-            const int64_t sp = (int64_t)a.list[rg.x + b_start + j] - vbase;
-            if (!FSS_CHECKED(sp >= 0 && sp < P.N)) continue;  // recorded by the staging loop
-            const int slot = a.splat_slot[sp];
-            if (!in_bounds(a.st, SITE_SLOT, slot, P.N)) continue;
-            float* dst = a.grad_item + ((int64_t)view * P.N + slot) * GRAD_STRIDE;
-            red_add_v4(dst, v[0], v[1], v[2], v[3]);
-            red_add_v4(dst + 4, v[4], v[5], v[6], v[7]);
-            red_add_v4(dst + 8, v[8], v[9], v[10], v[11]);
-            if (VAR)
-                red_add_v4(dst + 12, v[12], v[13], v[14], 0.0f);  // colour b, projected-centre gradient
-            else
-                atomicAdd(dst + 12, v[12]);
-        }
-        {
-            const int c4 = C / 4;
-            for (int idx = tid; idx < cnt * c4; idx += NT) {
-                const int j = idx / c4, q = idx - j * c4;
-                const float* v = s_gf + j * C + 4 * q;
-                if (v[0] == 0.0f && v[1] == 0.0f && v[2] == 0.0f && v[3] == 0.0f) continue;
-                const int64_t sp = (int64_t)a.list[rg.x + b_start + j] - vbase;
-                if (!FSS_CHECKED(sp >= 0 && sp < P.N)) continue;  // recorded by the staging loop
-                const int slot = a.splat_slot[sp];
-                if (!in_bounds(a.st, SITE_SLOT, slot, P.N)) continue;
-                red_add_v4(a.feat_acc + (int64_t)slot * C + 4 * q, v[0], v[1], v[2], v[3]);
-            }
-        }
-    }
-    __syncthreads();
-    }  // tiles
-}
-
-// ---------------------------------------------------------------------------
 // k_bwd_geo_topk: back-to-front replay of the Top-K render, one warp per 8 x 4
 // pixel block, each warp on its own
 // ---------------------------------------------------------------------------
@@ -651,7 +432,7 @@ constexpr int GEO_THREADS = 128;  // threads per CTA (64 for 8 x 8 tiles): parts
 // any of the warp's pixels selected.  The feature kernel, which groups K entries
 // per pixel by surfel in shared memory first, and its dots in memory are then not
 // needed: 1296 x 968, 16 channels, K = 24 FP32 geometry and features 860 us
-// before, 555 here (step 1573 / 1264).  Bound by instruction issue: 16 selects and
+// before, 546 here (step 1573 / 1264).  Bound by instruction issue: 16 selects and
 // multiplies and 17 shuffles per surfel and warp for 16 channels.
 template <int CF, typename FT>
 struct GeoStage {
@@ -902,6 +683,255 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
         }
         cp_async_wait_all();
         __syncwarp();  // before the warp's next block
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_bwd_geo_full: the same replay for the full accumulation (K = 0)
+// ---------------------------------------------------------------------------
+// Every contributor takes the dot c_j . dL/dF and gives w dL/dF to its row.  The
+// block's dL/dF stays in registers for the whole walk, as PX pixels x 4 NQ channels
+// per lane (FullLanes: 8 x 8 at 64 channels), and serves both products: a lane's
+// partial dots of its PX pixels are reduce-scattered over the CL lanes that share
+// them, which leaves each lane its own pixel's dot (7 shuffles for 8 pixels); with the
+// block's weights from shared memory a lane's channel sums are reduce-scattered over the
+// pixel groups and added to the surfel's row in L2 (256 consecutive bytes a warp at 64
+// channels).  The next surfel's row is read ahead.  640 x 480, 500k surfels, 64 channels
+// FP32: 481 us with a CTA per tile, all channels of a pixel in its lane and 95
+// shuffles per surfel for the sums, 246 here; the step with 16 channels 421 -> 339, 128
+// channels (spilled there) 2609 -> 811.  Bound by instruction issue.
+struct FullGeoStage {
+    WarpStage st[2];
+    int32_t slot[2][32], sp[2][32];  // gradient slots and ids of the staged surfels
+    float4 w[2][8];                  // the block's weights of a surfel, two surfels in turn
+};
+
+__device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(addr), "f"(a), "f"(b) : "memory");
+}
+
+template <int TS, int CMAX, typename FT, bool VAR>
+__global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) / full_threads<TS>())
+    k_bwd_geo_full(const __grid_constant__ Cams cams, const __grid_constant__ RParams P, const BwdArgs a) {
+    using L = FullLanes<CMAX>;
+    constexpr int NT = full_threads<TS>(), NW = NT / 32, PARTS = TS * TS / NT, PX = L::PX, NQ = L::NQ, CL = L::CL;
+    constexpr unsigned ALL = 0xffffffffu;
+    __shared__ __align__(16) FullGeoStage s_stage[NW];
+    __shared__ int s_work;
+    if (a.st->err) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cl = lane % CL, pg = lane / CL;  // this lane's channels and pixels of the products
+    FullGeoStage& G = s_stage[warp];
+    const FT* __restrict__ feats = reinterpret_cast<const FT*>(a.feats);
+    const int C = P.C, total = cams.total_tiles * PARTS;
+    for (bool first = true;; first = false) {
+        int u;  // this CTA's next part of a tile (heavy tiles first)
+        if (!a.persistent) {
+            u = first ? (int)blockIdx.x : INT_MAX;
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) s_work = (int)atomicAdd(&a.st->work_geo, 1u);
+            __syncthreads();
+            u = s_work;
+        }
+        if (u >= total) return;
+        const int t = cams.tile_order ? cams.tile_order[u / PARTS] : u / PARTS;
+        const int wb = (u % PARTS) * NW + warp;  // this warp's block of the tile
+        const uint32_t wbit = 1u << wb;
+        const int view = view_of_tile(cams, t);
+        const CamDev& cam = cams.c[view];
+        const int lt = t - cam.tile_off;
+        const int tx = lt % cam.tiles_x, ty = lt / cam.tiles_x;
+        const int bx = tx * TS + 8 * (wb % (TS / 8)), by = ty * TS + 4 * (wb / (TS / 8));
+        const int px = bx + (lane & 7), py = by + (lane >> 3);
+        const bool inside = px < cam.W && py < cam.H;
+        const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
+        const int2 rg = checked_range(a.ranges, t, P.pair_cap, a.st);
+        const int64_t vbase = (int64_t)view * P.N;
+        // VAR instances carry the variants (spherical-harmonic item colours, low-pass filter)
+        const float* __restrict__ rgbv = a.rgb + (VAR && P.color_sh ? 3 * vbase : 0);
+        const int64_t pix = cam.pix_off + (int64_t)py * cam.W + px;
+        const uint32_t* list = a.list + rg.x;
+        const uint32_t* masks = a.masks + rg.x;
+        float* grows = a.grad_item + vbase * GRAD_STRIDE;  // this view's gradient rows
+
+        int nstop = 0;
+        float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
+        if (inside) {
+            nstop = min(a.saved_nstop[pix], rg.y - rg.x);
+            T = a.out_T[pix];
+            gr = a.d_rgb[3 * pix];
+            gg = a.d_rgb[3 * pix + 1];
+            gb = a.d_rgb[3 * pix + 2];
+            Sh = P.bg[0] * gr + P.bg[1] * gg + P.bg[2] * gb + (a.d_T ? a.d_T[pix] : 0.0f);
+        }
+        const int len = __reduce_max_sync(ALL, nstop);
+        if (len == 0) continue;
+        float2 df[PX][NQ][2];  // the lane's pixels x channels of dL/dF
+#pragma unroll
+        for (int p = 0; p < PX; ++p) {
+            const int i = pg * PX + p, qx = bx + (i & 7), qy = by + (i >> 3);
+            float4 f[NQ];
+            L::load_row(reinterpret_cast<const FT*>(a.d_feat) + (cam.pix_off + (int64_t)qy * cam.W + qx) * C, cl,
+                        qx < cam.W && qy < cam.H ? C : 0, f);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                df[p][q][0] = make_float2(f[q].x, f[q].y);
+                df[p][q][1] = make_float2(f[q].z, f[q].w);
+            }
+        }
+
+        // one chunk's records and gradient slots, and the lane mask of those the warp meets
+        auto stage = [&](int buf, const ListEntry& e) {
+            const int64_t sp = (int64_t)e.item - vbase;
+            if ((e.mask & wbit) && FSS_CHECKED(sp >= 0 && sp < P.N)) {
+                cp_async4(&G.slot[buf][lane], a.splat_slot + sp);
+                G.sp[buf][lane] = (int32_t)sp;
+            }
+            return stage_chunk(G.st[buf], e, wbit, a.rec, rgbv, vbase, P.N, a.st);
+        };
+        // chunk b0 is worked on while the one before it is copied and the list entries of the next are read
+        int b0 = ((len - 1) >> 5) << 5;
+        ListEntry e1 = list_entry(list, masks, b0 + lane, len);
+        uint32_t word = stage((b0 >> 5) & 1, e1);
+        e1 = list_entry(list, masks, b0 - 32 + lane, len);
+        int par = 0;
+        for (; b0 >= 0; b0 -= 32) {
+            const int buf = (b0 >> 5) & 1;
+            const WarpStage& S = G.st[buf];
+            const uint32_t next = stage(buf ^ 1, e1);
+            e1 = list_entry(list, masks, b0 - 64 + lane, len);
+            cp_async_wait_prev();  // this chunk's copies
+            __syncwarp();
+            float4 nf[NQ];
+            if (word) L::load_row(feats + (int64_t)G.sp[buf][31 - __clz(word)] * C, cl, C, nf);
+            for (uint32_t bits = word; bits != 0u;) {
+                const int j = 31 - __clz(bits), pos = b0 + j;
+                bits ^= 0x80000000u >> __clz(bits);
+                float4 f[NQ];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) f[q] = nf[q];
+                if (bits) L::load_row(feats + (int64_t)G.sp[buf][31 - __clz(bits)] * C, cl, C, nf);
+                Hit h;
+                const float4 oc = S.oc[j];
+                const bool contrib = pos < nstop && eval_splat<VAR>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf, P.alpha_min,
+                                                                    cam.near_plane, h, P.lowpass);
+                if (!__any_sync(ALL, contrib)) continue;
+                // c_j . dL/dF, this lane's pixel
+                float dot[PX];
+#pragma unroll
+                for (int p = 0; p < PX; ++p) {
+                    float2 d = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        d = __ffma2_rn(make_float2(f[q].x, f[q].y), df[p][q][0], d);
+                        d = __ffma2_rn(make_float2(f[q].z, f[q].w), df[p][q][1], d);
+                    }
+                    dot[p] = d.x + d.y;
+                }
+#pragma unroll
+                for (int o = CL / 2, n = PX / 2; o > 0; o >>= 1, n >>= 1) {
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int i = 0; i < n; ++i) {
+                        const float send = up ? dot[i] : dot[i + n];
+                        const float keep = up ? dot[i + n] : dot[i];
+                        dot[i] = keep + __shfl_xor_sync(ALL, send, o);
+                    }
+                }
+                float g[VAR ? 16 : 13];
+#pragma unroll
+                for (int k = 0; k < (VAR ? 16 : 13); ++k) g[k] = 0.0f;
+                float w = 0.0f;
+                if (contrib) {
+                    const float alpha = fminf(h.alpha_raw, P.alpha_max);
+                    const float Tj = T * rcp_approx(1.0f - alpha);
+                    w = alpha * Tj;
+                    const float s = oc.y * gr + oc.z * gg + oc.w * gb + dot[0];
+                    const float dal = Tj * (s - Sh);
+                    Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
+                    g[10] = w * gr;
+                    g[11] = w * gg;
+                    g[12] = w * gb;
+                    if (h.alpha_raw < P.alpha_max) {
+                        g[9] = dal * h.G;
+                        const float drho = -0.5f * alpha * dal;
+                        if (VAR && h.scr) {  // low-pass screen term: rho = 2 |x - c|^2, d rho / d c = -4 (X, Y)
+                            g[VAR ? 13 : 0] = -4.0f * h.X * drho;
+                            g[VAR ? 14 : 0] = -4.0f * h.Y * drho;
+                        } else {
+                            const float du = 2.0f * h.u * drho, dv = 2.0f * h.v * drho;
+                            const float gc0 = du * h.inv, gc1 = dv * h.inv, gc2 = -(du * h.u + dv * h.v) * h.inv;
+                            g[0] = gc0 * h.X; g[1] = gc0 * h.Y; g[2] = gc0;
+                            g[3] = gc1 * h.X; g[4] = gc1 * h.Y; g[5] = gc1;
+                            g[6] = gc2 * h.X; g[7] = gc2 * h.Y; g[8] = gc2;
+                        }
+                    }
+                    T = Tj;
+                }
+                reinterpret_cast<float*>(G.w[par])[lane] = w;
+                if constexpr (VAR) reduce_scatter<16>(g);  // lane l holds value l >> 1
+                else reduce_scatter13(g);
+                const int slot = G.slot[buf][j];
+                const bool slot_ok = in_bounds(a.st, SITE_SLOT, slot, P.N);
+                if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13) && slot_ok)
+                    atomicAdd(grows + (int64_t)slot * GRAD_STRIDE + (lane >> 1), g[0]);
+                // w dL/dF: the sum over the lane's pixels, then over the pixel groups
+                __syncwarp();
+                float wp[PX], gf[4 * NQ];
+                L::load_weights(reinterpret_cast<const float*>(G.w[par]) + pg * PX, wp);
+                par ^= 1;
+                {
+                    float2 sum[NQ][2];
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) sum[q][0] = sum[q][1] = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int p = 0; p < PX; ++p)
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                            for (int k = 0; k < 2; ++k)
+                                sum[q][k] = __ffma2_rn(make_float2(wp[p], wp[p]), df[p][q][k], sum[q][k]);
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        gf[4 * q] = sum[q][0].x;
+                        gf[4 * q + 1] = sum[q][0].y;
+                        gf[4 * q + 2] = sum[q][1].x;
+                        gf[4 * q + 3] = sum[q][1].y;
+                    }
+                }
+                int n = 4 * NQ;
+#pragma unroll
+                for (int o = 16; o >= CL; o >>= 1) {
+                    if (n > 1) {
+                        const bool up = (lane & o) != 0;
+#pragma unroll
+                        for (int i = 0; i < 2 * NQ; ++i) {
+                            if (i < n / 2) {
+                                const float send = up ? gf[i] : gf[i + n / 2];
+                                const float keep = up ? gf[i + n / 2] : gf[i];
+                                gf[i] = keep + __shfl_xor_sync(ALL, send, o);
+                            }
+                        }
+                        n >>= 1;
+                    } else {
+                        gf[0] += __shfl_xor_sync(ALL, gf[0], o);
+                    }
+                }
+                // the lane's NQ sums are those of its values (lane >> 3) NQ on, consecutive channels
+                const int v0 = (lane >> 3) * NQ, c = 4 * (cl + CL * (v0 >> 2)) + (v0 & 3);
+                if (c < C && slot_ok && (CL == 8 || (lane & 4) == 0)) {
+                    float* dst = a.feat_acc + (int64_t)slot * C + c;
+                    if constexpr (NQ == 4) red_add_v4(dst, gf[0], gf[1], gf[2], gf[3]);
+                    else if constexpr (NQ == 2) red_add_v2(dst, gf[0], gf[1]);
+                    else atomicAdd(dst, gf[0]);
+                }
+            }
+            word = next;
+            __syncwarp();  // every lane has read this half before the next copies into it
+        }
+        cp_async_wait_all();
+        __syncwarp();
     }
 }
 
@@ -1201,16 +1231,16 @@ cudaError_t launch_feat(const Cams& cams, const RParams& P, const BwdArgs& a, cu
 
 template <int TS, int CMAX, typename FT, bool VAR>
 cudaError_t launch_geo_full(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
-    constexpr int NB = FBATCH;
-    const size_t smem = (size_t)NB * (4 * 16 + 8) + (size_t)NB * 16 * 4 + (size_t)NB * P.C * 8;  // staging, masks, partials, rows
-    cudaError_t e = set_smem((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR>, smem);
-    if (e != cudaSuccess) return e;
-    int grid = cams.total_tiles;
-    if (a.persistent &&
-        (e = persistent_grid((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR>, TS * TS, smem, grid)) != cudaSuccess)
-        return e;
-    k_bwd_geo_full<TS, CMAX, FT, VAR><<<grid, TS * TS, smem, s>>>(cams, P, a);
-    e = cudaGetLastError();
+    constexpr int NT = full_threads<TS>();
+    int64_t units = (int64_t)cams.total_tiles * (TS * TS / NT);
+    if (a.persistent) {
+        int wave = (int)std::min<int64_t>(units, INT_MAX);
+        const cudaError_t e = persistent_grid((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR>, NT, 0, wave);
+        if (e != cudaSuccess) return e;
+        units = wave;
+    }
+    k_bwd_geo_full<TS, CMAX, FT, VAR><<<(unsigned)units, NT, 0, s>>>(cams, P, a);
+    const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) kernel_mark(s);
     return e;
 }
@@ -1255,6 +1285,7 @@ cudaError_t launch_geo(const Cams& cams, const RParams& P, const BwdArgs& a, cud
     // filter) have their own instances: no cost on the plain paths
     if (P.K > 0) return launch_geo_topk<TS, FT>(cams, P, a, s);
     const bool var = P.color_sh || P.lowpass;
+    if (P.C <= 16) return var ? launch_geo_full<TS, 16, FT, true>(cams, P, a, s) : launch_geo_full<TS, 16, FT, false>(cams, P, a, s);
     if (P.C <= 32) return var ? launch_geo_full<TS, 32, FT, true>(cams, P, a, s) : launch_geo_full<TS, 32, FT, false>(cams, P, a, s);
     if (P.C <= 64) return var ? launch_geo_full<TS, 64, FT, true>(cams, P, a, s) : launch_geo_full<TS, 64, FT, false>(cams, P, a, s);
     return var ? launch_geo_full<TS, 128, FT, true>(cams, P, a, s) : launch_geo_full<TS, 128, FT, false>(cams, P, a, s);
