@@ -405,7 +405,7 @@ fss_status fss_forward_static(const fss_params *params, const fss_camera *cams, 
  * the loss runs in the render kernel (else 2), fss_sort_render_forward_loss 1
  * when the loss runs in the render kernel (else 3), fss_render_backward 4 for Top-K
  * (clear, feature gradients, geometry replay, projection; where the replay
- * also takes the feature gradients, K > 8 with at most 32 channels, their event
+ * also takes the feature gradients, as with many channels and large K, their event
  * is recorded with no kernel before it) or 3 for K = 0,
  * plus 1 when g_feat is given (feature rows).
  */

@@ -17,8 +17,8 @@
 //             surfel the warp reduce-scatters its 13 partial derivatives
 //             (adjugate rows 9, opacity 1, colour 3) and adds them to the
 //             surfel's gradient row.
-// k_bwd_geo_full (K = 0) the same, with c_j . dL/dF and the feature gradients of
-//             every contributor as products shared by the warp's lanes.
+// k_bwd_geo_full (K = 0, and Top-K with many channels x K) the same, with c_j . dL/dF
+//             and the feature gradients as products shared by the warp's lanes.
 // k_bwd_project one thread per surfel: adjugate-row gradients -> homography
 //             columns -> means, scales, quaternions; sums the views.
 // k_feat_out  writes every row of the feature gradient (zeros for surfels
@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 namespace fss {
 
@@ -423,7 +424,6 @@ __global__ void __launch_bounds__(BWD_FEAT_THREADS, 4) k_bwd_feat(const __grid_c
 // 640 x 480 frame of 500k surfels, 88 here; 1296 x 968 with K = 24 324 / 305.
 // Bound by instruction issue: about 40 of a warp evaluation's instructions are
 // the record, the ray and the derivatives, 55 the reduce-scatter.
-constexpr int FEAT_IN_GEO_C = 32, FEAT_IN_GEO_K = 9;  // see feat_in_geo
 constexpr int GEO_THREADS = 128;  // threads per CTA (64 for 8 x 8 tiles): parts of a tile
 
 // CF > 0 instances (16 or 32: channels, rounded up) also take the feature
@@ -431,7 +431,7 @@ constexpr int GEO_THREADS = 128;  // threads per CTA (64 for 8 x 8 tiles): parts
 // gradient in registers, and one more reduce-scatter of w dL/dF per surfel that
 // any of the warp's pixels selected.  The feature kernel, which groups K entries
 // per pixel by surfel in shared memory first, and its dots in memory are then not
-// needed: 1296 x 968, 16 channels, K = 24 FP32 geometry and features 860 us
+// needed (which path: feat_path): 1296 x 968, 16 channels, K = 24 FP32 geometry and features 860 us
 // before, 546 here (step 1573 / 1264).  Bound by instruction issue: 16 selects and
 // multiplies and 17 shuffles per surfel and warp for 16 channels.
 template <int CF, typename FT>
@@ -689,6 +689,9 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
 // ---------------------------------------------------------------------------
 // k_bwd_geo_full: the same replay for the full accumulation (K = 0)
 // ---------------------------------------------------------------------------
+// (TOPK: only the selected contributors, with the forward's weights; a surfel that none
+// of the warp's pixels selected costs no products, and a dL/dF that is not finite makes the
+// block leave out the products of pixels that did not select the surfel.)
 // Every contributor takes the dot c_j . dL/dF and gives w dL/dF to its row.  The
 // block's dL/dF stays in registers for the whole walk, as PX pixels x 4 NQ channels
 // per lane (FullLanes: 8 x 8 at 64 channels), and serves both products: a lane's
@@ -710,7 +713,7 @@ __device__ __forceinline__ void red_add_v2(float* addr, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(addr), "f"(a), "f"(b) : "memory");
 }
 
-template <int TS, int CMAX, typename FT, bool VAR>
+template <int TS, int CMAX, typename FT, bool VAR, bool TOPK = false>
 __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) / full_threads<TS>())
     k_bwd_geo_full(const __grid_constant__ Cams cams, const __grid_constant__ RParams P, const BwdArgs a) {
     using L = FullLanes<CMAX>;
@@ -755,6 +758,9 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
         const uint32_t* masks = a.masks + rg.x;
         float* grows = a.grad_item + vbase * GRAD_STRIDE;  // this view's gradient rows
 
+        const int K = P.K;
+        int kk = -1, next_pos = -1;  // TOPK: the pixel's next selected surfel ...
+        float next_w = 0.0f;         // ... and the forward's weight of it
         int nstop = 0;
         float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
         if (inside) {
@@ -764,6 +770,14 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
             gg = a.d_rgb[3 * pix + 1];
             gb = a.d_rgb[3 * pix + 2];
             Sh = P.bg[0] * gr + P.bg[1] * gg + P.bg[2] * gb + (a.d_T ? a.d_T[pix] : 0.0f);
+            if constexpr (TOPK) {
+                for (kk = K - 1; kk >= 0; --kk)
+                    if (a.saved_pos[pix * K + kk] >= 0) break;
+                if (kk >= 0) {
+                    next_pos = a.saved_pos[pix * K + kk];
+                    next_w = a.saved_w[pix * K + kk];
+                }
+            }
         }
         const int len = __reduce_max_sync(ALL, nstop);
         if (len == 0) continue;
@@ -779,6 +793,17 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                 df[p][q][0] = make_float2(f[q].x, f[q].y);
                 df[p][q][1] = make_float2(f[q].z, f[q].w);
             }
+        }
+        bool careful = false;  // TOPK: some dL/dF is not finite
+        if constexpr (TOPK) {
+            float2 z = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int p = 0; p < PX; ++p)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) z = __ffma2_rn(df[p][q][k], make_float2(0.0f, 0.0f), z);
+            careful = __any_sync(ALL, !(z.x + z.y == 0.0f));
         }
 
         // one chunk's records and gradient slots, and the lane mask of those the warp meets
@@ -817,8 +842,11 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                 const bool contrib = pos < nstop && eval_splat<VAR>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf, P.alpha_min,
                                                                     cam.near_plane, h, P.lowpass);
                 if (!__any_sync(ALL, contrib)) continue;
+                const bool sel = TOPK ? contrib && pos == next_pos : contrib;
+                const bool feat = TOPK ? __any_sync(ALL, sel) : true;
                 // c_j . dL/dF, this lane's pixel
                 float dot[PX];
+                if (feat) {
 #pragma unroll
                 for (int p = 0; p < PX; ++p) {
                     float2 d = make_float2(0.0f, 0.0f);
@@ -839,15 +867,27 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                         dot[i] = keep + __shfl_xor_sync(ALL, send, o);
                     }
                 }
+                }
                 float g[VAR ? 16 : 13];
 #pragma unroll
                 for (int k = 0; k < (VAR ? 16 : 13); ++k) g[k] = 0.0f;
-                float w = 0.0f;
+                float w = 0.0f, wf = -0.0f;  // wf: the weight on dL/dF (-0: not one of its pixels)
                 if (contrib) {
                     const float alpha = fminf(h.alpha_raw, P.alpha_max);
                     const float Tj = T * rcp_approx(1.0f - alpha);
                     w = alpha * Tj;
-                    const float s = oc.y * gr + oc.z * gg + oc.w * gb + dot[0];
+                    float s = oc.y * gr + oc.z * gg + oc.w * gb;
+                    if (sel) s += dot[0];
+                    if constexpr (TOPK) {
+                        if (sel) {
+                            wf = next_w;
+                            --kk;
+                            next_pos = kk >= 0 ? a.saved_pos[pix * K + kk] : -1;
+                            next_w = kk >= 0 ? a.saved_w[pix * K + kk] : 0.0f;
+                        }
+                    } else {
+                        wf = w;
+                    }
                     const float dal = Tj * (s - Sh);
                     Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
                     g[10] = w * gr;
@@ -869,13 +909,14 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                     }
                     T = Tj;
                 }
-                reinterpret_cast<float*>(G.w[par])[lane] = w;
+                if (feat) reinterpret_cast<float*>(G.w[par])[lane] = wf;
                 if constexpr (VAR) reduce_scatter<16>(g);  // lane l holds value l >> 1
                 else reduce_scatter13(g);
                 const int slot = G.slot[buf][j];
                 const bool slot_ok = in_bounds(a.st, SITE_SLOT, slot, P.N);
                 if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13) && slot_ok)
                     atomicAdd(grows + (int64_t)slot * GRAD_STRIDE + (lane >> 1), g[0]);
+                if (!feat) continue;
                 // w dL/dF: the sum over the lane's pixels, then over the pixel groups
                 __syncwarp();
                 float wp[PX], gf[4 * NQ];
@@ -885,13 +926,19 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                     float2 sum[NQ][2];
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) sum[q][0] = sum[q][1] = make_float2(0.0f, 0.0f);
+                    auto pixels = [&](auto select) {
 #pragma unroll
-                    for (int p = 0; p < PX; ++p)
+                        for (int p = 0; p < PX; ++p) {
+                            if (decltype(select)::value && __float_as_uint(wp[p]) == 0x80000000u) continue;
 #pragma unroll
-                        for (int q = 0; q < NQ; ++q)
+                            for (int q = 0; q < NQ; ++q)
 #pragma unroll
-                            for (int k = 0; k < 2; ++k)
-                                sum[q][k] = __ffma2_rn(make_float2(wp[p], wp[p]), df[p][q][k], sum[q][k]);
+                                for (int k = 0; k < 2; ++k)
+                                    sum[q][k] = __ffma2_rn(make_float2(wp[p], wp[p]), df[p][q][k], sum[q][k]);
+                        }
+                    };
+                    if (TOPK && careful) pixels(std::true_type{});
+                    else pixels(std::false_type{});
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
                         gf[4 * q] = sum[q][0].x;
@@ -1229,36 +1276,59 @@ cudaError_t launch_feat(const Cams& cams, const RParams& P, const BwdArgs& a, cu
     }
 }
 
-template <int TS, int CMAX, typename FT, bool VAR>
+template <int TS, int CMAX, typename FT, bool VAR, bool TOPK = false>
 cudaError_t launch_geo_full(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
     constexpr int NT = full_threads<TS>();
     int64_t units = (int64_t)cams.total_tiles * (TS * TS / NT);
     if (a.persistent) {
         int wave = (int)std::min<int64_t>(units, INT_MAX);
-        const cudaError_t e = persistent_grid((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR>, NT, 0, wave);
+        const cudaError_t e = persistent_grid((const void*)k_bwd_geo_full<TS, CMAX, FT, VAR, TOPK>, NT, 0, wave);
         if (e != cudaSuccess) return e;
         units = wave;
     }
-    k_bwd_geo_full<TS, CMAX, FT, VAR><<<(unsigned)units, NT, 0, s>>>(cams, P, a);
+    k_bwd_geo_full<TS, CMAX, FT, VAR, TOPK><<<(unsigned)units, NT, 0, s>>>(cams, P, a);
     const cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) kernel_mark(s);
     return e;
 }
 
-// The feature gradients in the replay kernel: the feature kernel's work grows
-// with K, the replay's little.  640 x 480 steps, feature kernel / replay: 16
-// channels FP32 K = 8 196 / 187 us (but the feature rows then no longer run
-// beside the replay when launched eagerly: level), K = 9 242 / 222, K = 32 401 /
-// 300; 32 channels FP32 K = 8 224 / 230, K = 9 278 / 269, K = 32 455 / 380, BF16
-// K = 8 207 / 215, K = 9 254 / 247; 24 channels, 1296 x 968, tiles of 8, 16, 32, K = 16 1.04
-// to 1.17x.  Not with a renormalised selection, which needs every dot before the
-// first, nor with the other variants.
-bool feat_in_geo(const RParams& P) {
-    return P.K >= FEAT_IN_GEO_K && P.C <= FEAT_IN_GEO_C && !P.renorm && !P.color_sh && !P.lowpass;
+// Who takes the feature gradients of a Top-K backward.  The feature kernel's work
+// grows with K, the replay kernels' little, and theirs does not shrink with BF16 as the
+// feature kernel's does.  Training steps, us, feature kernel / replay:
+// k_bwd_geo_topk (16 and, BF16, 32 channels), 640 x 480: 16 channels FP32 K = 8 196 /
+//   187 (but the feature rows then no longer run beside the replay when launched
+//   eagerly: level), K = 9 242 / 222, K = 32 401 / 300; 32 channels BF16 K = 8 207 /
+//   215, K = 9 254 / 247, K = 32 425 / 327.
+// k_bwd_geo_full (instances of 32, 64 and 128 channels, whose cost does not fall with fewer):
+//   640 x 480 FP32: 64 channels K = 4 268 / 244, K = 8 307 / 264, K = 32 568 / 420; 128
+//   channels K = 8 463 / 395, K = 32 798 / 634, but 72 channels K = 4 345 / 368; BF16 64
+//   channels K = 8 243 / 249, K = 24 434 / 351, but 128 channels K = 16 464 / 473.  With
+//   more and smaller surfels (800k, 1280 x 720, exact stop): FP32 40 channels K = 4 691 /
+//   711, 64 K = 4 776 / 762 (640 x 360, tiles of 8: 349 / 353), K = 8 955 / 906, 72 K = 8
+//   1154 / 1219 (K = 16 605 / 628), 112 K = 12 1845 / 1775; BF16 64 K = 16 1249 / 1285, 48 K = 24 1722 / 1621.  So by channels x K.  Against
+//   k_bwd_geo_topk: FP32 32 channels K = 24 337 / 303, 24 K = 12 985 / 960, 16 channels
+//   level; BF16 16 channels 248 / 261, 32 298 / 288 but on small images 220 / 241.
+//   A warp on its own has a long chain per surfel: with few 8 x 4 blocks an SM the feature
+//   kernel's more threads are ahead (tiles of 8: 128 x 128, 64 channels K = 8 FP32 172 /
+//   188, 200 x 150 117 / 116; of 16: 64 x 48 533 / 548, 128 x 128 FP32 197 / 189, BF16
+//   183 / 199; of 32: 128 x 128 443 / 334).
+// Neither with a renormalised selection, which needs every dot before the first, nor with
+// the other variants.
+enum FeatPath { FEAT_KERNEL, FEAT_REPLAY, FEAT_PRODUCTS };
+FeatPath feat_path(const Cams& cams, const RParams& P, int num_sms) {
+    if (P.K == 0 || P.renorm || P.color_sh || P.lowpass) return FEAT_KERNEL;
+    const bool half = P.feat_dtype == FSS_BF16;
+    if (P.K > 8 && P.C <= (half ? 32 : 16)) return FEAT_REPLAY;
+    const int64_t blocks = (int64_t)cams.total_tiles * (P.ts * P.ts / 32);
+    if (blocks >= (int64_t)num_sms * (P.ts == 8 ? 8 : P.ts == 16 ? (half ? 4 : 2) : 0) &&
+        (half ? P.C > 32 && P.C <= 64 && P.C * P.K >= 1152
+              : P.C > 16 && P.C <= 128 && P.C * P.K >= (P.C <= 64 ? 288 : 1200) && (P.C > 32 || P.K > 8)))
+        return FEAT_PRODUCTS;
+    return P.K > 8 && P.C <= 32 ? FEAT_REPLAY : FEAT_KERNEL;
 }
 
 template <int TS, typename FT>
-cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
+cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a, FeatPath feat, cudaStream_t s) {
     auto go = [&](auto kern, int nt) {
         int64_t units = (int64_t)cams.total_tiles * (TS * TS / nt);
         if (a.persistent) {
@@ -1272,7 +1342,14 @@ cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a
         if (e == cudaSuccess) kernel_mark(s);
         return e;
     };
-    if (feat_in_geo(P))
+    if (feat == FEAT_PRODUCTS) {
+        if (P.C <= 32) {
+            if constexpr (sizeof(FT) == 4) return launch_geo_full<TS, 32, FT, false, true>(cams, P, a, s);
+        }
+        if (P.C <= 64) return launch_geo_full<TS, 64, FT, false, true>(cams, P, a, s);
+        if constexpr (sizeof(FT) == 4) return launch_geo_full<TS, 128, FT, false, true>(cams, P, a, s);
+    }
+    if (feat == FEAT_REPLAY)
         return P.C <= 16 ? go(k_bwd_geo_topk<TS, false, 16, FT>, geo_threads<TS, 16, FT>())
                          : go(k_bwd_geo_topk<TS, false, 32, FT>, geo_threads<TS, 32, FT>());
     return P.renorm || P.color_sh || P.lowpass ? go(k_bwd_geo_topk<TS, true>, geo_threads<TS, 0, float>())
@@ -1280,10 +1357,10 @@ cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a
 }
 
 template <int TS, typename FT>
-cudaError_t launch_geo(const Cams& cams, const RParams& P, const BwdArgs& a, cudaStream_t s) {
+cudaError_t launch_geo(const Cams& cams, const RParams& P, const BwdArgs& a, FeatPath feat, cudaStream_t s) {
     // the variants (renormalised Top-K, spherical-harmonic colours, low-pass
     // filter) have their own instances: no cost on the plain paths
-    if (P.K > 0) return launch_geo_topk<TS, FT>(cams, P, a, s);
+    if (P.K > 0) return launch_geo_topk<TS, FT>(cams, P, a, feat, s);
     const bool var = P.color_sh || P.lowpass;
     if (P.C <= 16) return var ? launch_geo_full<TS, 16, FT, true>(cams, P, a, s) : launch_geo_full<TS, 16, FT, false>(cams, P, a, s);
     if (P.C <= 32) return var ? launch_geo_full<TS, 32, FT, true>(cams, P, a, s) : launch_geo_full<TS, 32, FT, false>(cams, P, a, s);
@@ -1298,7 +1375,8 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     k_bwd_clear<<<num_sms * 4, 256, 0, s>>>(cams, P, a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     kernel_mark(s);
-    if (feat_in_geo(P)) {
+    const FeatPath feat = feat_path(cams, P, num_sms);
+    if (P.K > 0 && feat != FEAT_KERNEL) {
         kernel_mark(s);  // the feature gradients' place among the events: nothing runs there
     } else if (P.K > 0) {
         if ((e = launch_feat<FT>(cams, P, a, s)) != cudaSuccess) return e;
@@ -1312,7 +1390,7 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return e;
-    const bool fork = a.g_feat && P.K > 0 && !feat_in_geo(P) && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
+    const bool fork = a.g_feat && P.K > 0 && feat == FEAT_KERNEL && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
                       side_stream(s, side, ev_fork, ev_join);
     if (fork) {
         if ((e = cudaEventRecord(ev_fork, s)) != cudaSuccess) return e;
@@ -1333,9 +1411,9 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
         }
         return err;
     };
-    if (P.ts == 8) e = launch_geo<8, FT>(cams, P, a, s);
-    else if (P.ts == 16) e = launch_geo<16, FT>(cams, P, a, s);
-    else e = launch_geo<32, FT>(cams, P, a, s);
+    if (P.ts == 8) e = launch_geo<8, FT>(cams, P, a, feat, s);
+    else if (P.ts == 16) e = launch_geo<16, FT>(cams, P, a, feat, s);
+    else e = launch_geo<32, FT>(cams, P, a, feat, s);
     if (e != cudaSuccess) return joined(e);
     const int64_t nb = (P.N + 255) / 256;
     // the coefficient gradients' zeros as one memset: written by each surfel's

@@ -20,17 +20,19 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("C,dtype,K,ts", [
     (4, torch.float32, 9, 16), (12, torch.float32, 16, 8), (16, torch.float32, 24, 16), (20, torch.float32, 10, 32),
     (32, torch.float32, 32, 16), (36, torch.float32, 9, 16), (8, torch.bfloat16, 9, 16), (16, torch.bfloat16, 17, 32),
-    (24, torch.bfloat16, 12, 8), (32, torch.bfloat16, 24, 16), (16, torch.float32, 8, 16)])
+    (24, torch.bfloat16, 12, 8), (32, torch.bfloat16, 24, 16), (16, torch.float32, 8, 16),
+    (20, torch.float32, 9, 32), (36, torch.float32, 8, 32), (64, torch.float32, 16, 32), (68, torch.float32, 17, 32),
+    (128, torch.float32, 32, 32), (40, torch.bfloat16, 32, 32), (64, torch.bfloat16, 24, 32), (64, torch.float32, 3, 32)])
 def test_feature_gradients_in_the_replay(C, dtype, K, ts):
     sc, cam = scenes.tiny_scene(seed=51 + C, n=1200, C=C)
     sc.opacities *= np.float32(0.3)
     _check(sc, cam, K, dtype, tile_size=ts, seed=C + K)
 
 
-@pytest.mark.parametrize("C", [16, 32])
+@pytest.mark.parametrize("C", [16, 32, 64])
 def test_an_infinite_gradient_stays_with_its_surfels(C):
     sc, cam = scenes.tiny_scene(seed=5, n=1200, C=C)
-    run = GpuRun(sc, [cam], K=12, tile_size=16, feat_dtype=torch.float32)
+    run = GpuRun(sc, [cam], K=12, tile_size=32, feat_dtype=torch.float32)
     ids = np.asarray(run.view(0)["ids"])
     H, W = ids.shape[:2]
     gF = np.ones((H, W, C))
