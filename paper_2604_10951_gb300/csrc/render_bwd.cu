@@ -1381,18 +1381,20 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     } else if (P.K > 0) {
         if ((e = launch_feat<FT>(cams, P, a, s)) != cudaSuccess) return e;
     }
-    // With Top-K the feature gradients are complete here: launched eagerly,
-    // their output pass (memory bound) runs in a second stream beside the
-    // geometry replay (issue bound) and joins before the call returns: 10 us
-    // less per 500k-surfel frame.  A graph being captured keeps one stream:
-    // replayed, the branch measured 3 us slower than the chain.
+    // Once the feature gradients are complete their output pass (memory bound)
+    // runs in a second stream, launched eagerly, beside the geometry replay
+    // (issue bound; 10 us less per 500k-surfel frame) or, where the replay took
+    // them, beside the projection, and joins before the call returns.  A graph
+    // being captured keeps one stream: replayed, the branch measured 3 us slower
+    // than the chain.
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return e;
-    const bool fork = a.g_feat && P.K > 0 && feat == FEAT_KERNEL && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
+    const bool fork = a.g_feat && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
                       side_stream(s, side, ev_fork, ev_join);
-    if (fork) {
+    bool forked = false;
+    auto rows_beside = [&]() {
         if ((e = cudaEventRecord(ev_fork, s)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(side, ev_fork, 0)) != cudaSuccess) return e;
         k_feat_out<FT><<<num_sms * 8, 256, 0, side>>>(P, a);
@@ -1401,11 +1403,15 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
             (void)cudaStreamSynchronize(side);  // no join event: wait for the side stream's kernel here
             return e;
         }
-    }
+        forked = true;
+        return e;
+    };
+    const bool before = P.K > 0 && feat == FEAT_KERNEL;  // complete before the replay
+    if (fork && before && (e = rows_beside()) != cudaSuccess) return e;
     // from here on every return joins the side stream first, so that no work of
     // this call is left running after it returns, even on an error
     auto joined = [&](cudaError_t err) {
-        if (fork) {
+        if (forked) {
             const cudaError_t ej = cudaStreamWaitEvent(s, ev_join, 0);
             if (err == cudaSuccess) err = ej;
         }
@@ -1415,6 +1421,7 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     else if (P.ts == 16) e = launch_geo<16, FT>(cams, P, a, feat, s);
     else e = launch_geo<32, FT>(cams, P, a, feat, s);
     if (e != cudaSuccess) return joined(e);
+    if (fork && !before && (e = rows_beside()) != cudaSuccess) return e;
     const int64_t nb = (P.N + 255) / 256;
     // the coefficient gradients' zeros as one memset: written by each surfel's
     // thread, 4 bytes at a time and a row apart, they took 70 of the projection's
