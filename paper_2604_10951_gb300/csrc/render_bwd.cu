@@ -426,14 +426,23 @@ __global__ void __launch_bounds__(BWD_FEAT_THREADS, 4) k_bwd_feat(const __grid_c
 // the record, the ray and the derivatives, 55 the reduce-scatter.
 constexpr int GEO_THREADS = 128;  // threads per CTA (64 for 8 x 8 tiles): parts of a tile
 
-// CF > 0 instances (16 or 32: channels, rounded up) also take the feature
-// gradients: the dot c_j . dL/dF from the surfel's staged row and the pixel's
-// gradient in registers, and one more reduce-scatter of w dL/dF per surfel that
-// any of the warp's pixels selected.  The feature kernel, which groups K entries
-// per pixel by surfel in shared memory first, and its dots in memory are then not
-// needed (which path: feat_path): 1296 x 968, 16 channels, K = 24 FP32 geometry and features 860 us
-// before, 546 here (step 1573 / 1264).  Bound by instruction issue: 16 selects and
-// multiplies and 17 shuffles per surfel and warp for 16 channels.
+// CF > 0 instances (16 or 32: channels, rounded up; which path: feat_path) also
+// take the feature gradients: the dot c_j . dL/dF from the surfel's staged row
+// and the pixel's gradient in registers, and one more reduce-scatter of w dL/dF
+// per surfel that any of the warp's pixels selected.  The feature kernel, which
+// groups K entries per pixel by surfel in shared memory first, and its dots in
+// memory are then not needed: 1296 x 968, 16 channels, K = 24 FP32 geometry and
+// features 860 us before, 546 with H = 1 (step 1573 / 1264).  Bound by
+// instruction issue: 16 selects and multiplies and 17 shuffles per surfel and
+// warp for 16 channels.
+// H = 2: a lane has a pixel of each of two blocks, one above the other, so a
+// surfel that meets both is read once and its sums go through one reduce-scatter
+// (1296 x 968, 500k surfels, 16 channels, K = 24: step FP32 1265 -> 1193 us, BF16
+// 1174 -> 1141; 640 x 480, K = 16 244 -> 237, BF16 level).  A warp then has twice the
+// work, which small images lose by (256 x 200 146 -> 170, 128 x 128 171 -> 215):
+// taken from 48 blocks an SM on.  Without the feature gradients it gains less than
+// it loses elsewhere: 1.2M surfels 1295 -> 1249, but six views of 1M 3206 -> 3217,
+// 640 x 480 328 -> 340.
 template <int CF, typename FT>
 struct GeoStage {
     WarpStage st[2];
@@ -442,10 +451,10 @@ struct GeoStage {
 };
 
 // threads per CTA: 64 where the stages of four warps are above 48 KB
-template <int TS, int CF, typename FT>
+template <int TS, int CF, typename FT, int H>
 constexpr int geo_threads() {
     const int nt = CF && 4 * sizeof(GeoStage<CF, FT>) > 47 * 1024 ? GEO_THREADS / 2 : GEO_THREADS;
-    return TS * TS < nt ? TS * TS : nt;
+    return TS * TS / H < nt ? TS * TS / H : nt;
 }
 
 // warp sums of v[0..12]: afterwards an even lane l < 26 holds the sum of v[l >> 1]
@@ -474,11 +483,11 @@ __device__ __forceinline__ void reduce_scatter13(float (&v)[13]) {
     v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-template <int TS, bool VAR, int CF = 0, typename FT = float>
-__global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
-                                  (CF == 0 ? 1024 : CF == 16 ? 768 : 512) / geo_threads<TS, CF, FT>())
+template <int TS, bool VAR, int CF = 0, typename FT = float, int H = 1>
+__global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
+                                  (CF == 0 ? 1024 : CF == 16 && H == 1 ? 768 : 512) / geo_threads<TS, CF, FT, H>())
     k_bwd_geo_topk(const __grid_constant__ Cams cams, const __grid_constant__ RParams P, const BwdArgs a) {
-    constexpr int NT = geo_threads<TS, CF, FT>(), NW = NT / 32, PARTS = TS * TS / NT;
+    constexpr int NT = geo_threads<TS, CF, FT, H>(), NW = NT / 32, PARTS = TS * TS / H / NT, WX = TS / 8;
     constexpr unsigned ALL = 0xffffffffu;
     static_assert(!VAR || CF == 0, "the variants take the feature gradients from their own kernel");
     __shared__ __align__(16) GeoStage<CF, FT> s_stage[NW];
@@ -506,69 +515,81 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
         }
         if (u >= total) return;
         const int t = cams.tile_order ? cams.tile_order[u / PARTS] : u / PARTS;
-        const int wb = (u % PARTS) * NW + warp;  // this warp's block of the tile
-        const uint32_t wbit = 1u << wb;
+        // this warp's block of the tile, or (H = 2) the upper one of two
+        const int wu = (u % PARTS) * NW + warp, wb = H == 2 ? 2 * WX * (wu / WX) + wu % WX : wu;
+        const uint32_t wbit = H == 2 ? (1u | 1u << WX) << wb : 1u << wb;
         const int view = view_of_tile(cams, t);
         const CamDev& cam = cams.c[view];
         const int lt = t - cam.tile_off;
         const int tx = lt % cam.tiles_x, ty = lt / cam.tiles_x;
-        const int px = tx * TS + 8 * (wb % (TS / 8)) + (lane & 7), py = ty * TS + 4 * (wb / (TS / 8)) + (lane >> 3);
-        const bool inside = px < cam.W && py < cam.H;
+        const int px = tx * TS + 8 * (wb % WX) + (lane & 7), py = ty * TS + 4 * (wb / WX) + (lane >> 3);
         const float pxf = (float)px + 0.5f, pyf = (float)py + 0.5f;
         const int2 rg = checked_range(a.ranges, t, P.pair_cap, a.st);
         const int64_t vbase = (int64_t)view * P.N;
         // VAR instances carry the variants (renormalised Top-K, spherical-harmonic
         // item colours, low-pass filter), read from the parameters
         const float* __restrict__ rgbv = a.rgb + (VAR && P.color_sh ? 3 * vbase : 0);
-        const int64_t pix = cam.pix_off + (int64_t)py * cam.W + px;
+        const int64_t pix0 = cam.pix_off + (int64_t)py * cam.W + px;
         const uint32_t* list = a.list + rg.x;
         const uint32_t* masks = a.masks + rg.x;
         float* grows = a.grad_item + vbase * GRAD_STRIDE;  // this view's gradient rows
 
-        int nstop = 0;
-        float T = 1.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f, Sh = 0.0f;
-        int kk = -1, next_pos = -1;
-        float next_dot = 0.0f;  // (CF: that surfel's weight)
+        int nstop[H], kk[H], next_pos[H], top = 0;
+        float T[H], gr[H], gg[H], gb[H], Sh[H];
+        float next_dot[H];  // (CF: that surfel's weight)
         // a selected surfel adds rn_a * dot + rn_b to what its weight multiplies:
         // the dot itself, or (dot - F.dL/dF) / W for the renormalised variant
-        float rn_a = 1.0f, rn_b = 0.0f;
-        if (inside) {
-            nstop = min(a.saved_nstop[pix], rg.y - rg.x);
-            T = a.out_T[pix];
-            gr = a.d_rgb[3 * pix];
-            gg = a.d_rgb[3 * pix + 1];
-            gb = a.d_rgb[3 * pix + 2];
-            Sh = P.bg[0] * gr + P.bg[1] * gg + P.bg[2] * gb + (a.d_T ? a.d_T[pix] : 0.0f);
-            for (kk = K - 1; kk >= 0; --kk)
-                if (a.saved_pos[pix * K + kk] >= 0) break;
-            if (kk >= 0) {
-                next_pos = a.saved_pos[pix * K + kk];
-                next_dot = (CF == 0 ? a.dots : a.saved_w)[pix * K + kk];
-            }
-            if (VAR && P.renorm) {  // entries 0..kk are the selected ones, front to back
-                float ws = 0.0f, wd = 0.0f;
-                for (int k2 = 0; k2 <= kk; ++k2) {
-                    const float wv = a.saved_w[pix * K + k2];
-                    ws += wv;
-                    wd = fmaf(wv, a.dots[pix * K + k2], wd);
+        float rn_a[H], rn_b[H];
+        float2 dfr[H][CF ? CF / 2 : 1];  // the pixels' dL/dF
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const int64_t pix = pix0 + (int64_t)(4 * i) * cam.W;
+            const bool inside = px < cam.W && py + 4 * i < cam.H;
+            nstop[i] = 0;
+            T[i] = 1.0f;
+            gr[i] = gg[i] = gb[i] = Sh[i] = next_dot[i] = rn_b[i] = 0.0f;
+            rn_a[i] = 1.0f;
+            kk[i] = next_pos[i] = -1;
+            if (inside) {
+                nstop[i] = min(a.saved_nstop[pix], rg.y - rg.x);
+                T[i] = a.out_T[pix];
+                gr[i] = a.d_rgb[3 * pix];
+                gg[i] = a.d_rgb[3 * pix + 1];
+                gb[i] = a.d_rgb[3 * pix + 2];
+                Sh[i] = P.bg[0] * gr[i] + P.bg[1] * gg[i] + P.bg[2] * gb[i] + (a.d_T ? a.d_T[pix] : 0.0f);
+                int k = K - 1;
+                for (; k >= 0; --k)
+                    if (a.saved_pos[pix * K + k] >= 0) break;
+                kk[i] = k;
+                if (k >= 0) {
+                    next_pos[i] = a.saved_pos[pix * K + k];
+                    next_dot[i] = (CF == 0 ? a.dots : a.saved_w)[pix * K + k];
                 }
-                rn_a = ws > 0.0f ? 1.0f / ws : 0.0f;
-                rn_b = -wd * rn_a * rn_a;
+                if (VAR && P.renorm) {  // entries 0..k are the selected ones, front to back
+                    float ws = 0.0f, wd = 0.0f;
+                    for (int k2 = 0; k2 <= k; ++k2) {
+                        const float wv = a.saved_w[pix * K + k2];
+                        ws += wv;
+                        wd = fmaf(wv, a.dots[pix * K + k2], wd);
+                    }
+                    rn_a[i] = ws > 0.0f ? 1.0f / ws : 0.0f;
+                    rn_b[i] = -wd * rn_a[i] * rn_a[i];
+                }
             }
-        }
-        float2 dfr[CF ? CF / 2 : 1];  // this pixel's dL/dF
-        if constexpr (CF > 0) {
+            if constexpr (CF > 0) {
 #pragma unroll
-            for (int v = 0; v < CF / E; ++v) {
-                float f[E];
+                for (int v = 0; v < CF / E; ++v) {
+                    float f[E];
 #pragma unroll
-                for (int e = 0; e < E; ++e) f[e] = 0.0f;
-                if (inside && v * E < P.C) FeatVec<FT>::load(reinterpret_cast<const FT*>(a.d_feat) + pix * P.C + v * E, f);
+                    for (int e = 0; e < E; ++e) f[e] = 0.0f;
+                    if (inside && v * E < P.C) FeatVec<FT>::load(reinterpret_cast<const FT*>(a.d_feat) + pix * P.C + v * E, f);
 #pragma unroll
-                for (int e = 0; e < E / 2; ++e) dfr[v * (E / 2) + e] = make_float2(f[2 * e], f[2 * e + 1]);
+                    for (int e = 0; e < E / 2; ++e) dfr[i][v * (E / 2) + e] = make_float2(f[2 * e], f[2 * e + 1]);
+                }
             }
+            top = max(top, nstop[i]);
         }
-        const int L = __reduce_max_sync(ALL, nstop);
+        const int L = __reduce_max_sync(ALL, top);
 
         // one chunk's records and gradient slots, and the lane mask of those the warp meets
         auto stage = [&](int buf, const ListEntry& e) {
@@ -586,12 +607,14 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
         // chunk b0 is worked on while the one before it is copied and the list entries of the next are read
         int b0 = ((L - 1) >> 5) << 5;  // (L = 0: the loop does not run)
         ListEntry e1 = list_entry(list, masks, b0 + lane, L);
-        uint32_t word = stage((b0 >> 5) & 1, e1);
+        uint32_t word = stage((b0 >> 5) & 1, e1), lower = 0u, lower_next = 0u;  // (H = 2: whose lower block is met)
+        if (H == 2) lower = __ballot_sync(ALL, (e1.mask & (1u << WX << wb)) != 0u);
         e1 = list_entry(list, masks, b0 - 32 + lane, L);
         for (; b0 >= 0 && L > 0; b0 -= 32) {
             const int buf = (b0 >> 5) & 1;
             const WarpStage& S = G.st[buf];
             const uint32_t next = stage(buf ^ 1, e1);
+            if (H == 2) lower_next = __ballot_sync(ALL, (e1.mask & (1u << WX << wb)) != 0u);
             e1 = list_entry(list, masks, b0 - 64 + lane, L);
             cp_async_wait_prev();  // this chunk's copies
             __syncwarp();
@@ -600,61 +623,74 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
                 float g[VAR ? 16 : 13];
 #pragma unroll
                 for (int k = 0; k < (VAR ? 16 : 13); ++k) g[k] = 0.0f;
-                bool contrib = false;
-                bool sel = false;  // CF: this pixel selected the surfel, with the forward's weight
-                float wsel = 0.0f;
-                Hit h;
+                bool contrib = false, sel[H];  // CF: this pixel selected the surfel, with the forward's weight
+                float wsel[H];
                 const float4 oc = S.oc[j];
-                if (pos < nstop &&
-                    eval_splat<VAR>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf, P.alpha_min, cam.near_plane, h, P.lowpass)) {
-                    contrib = true;
-                    const float alpha = fminf(h.alpha_raw, P.alpha_max);
-                    const float Tj = T * rcp_approx(1.0f - alpha);
-                    const float w = alpha * Tj;
-                    float s = oc.y * gr + oc.z * gg + oc.w * gb;
-                    if (pos == next_pos) {
-                        if constexpr (CF > 0) {
-                            float2 d0 = make_float2(0.0f, 0.0f), d1 = d0;
 #pragma unroll
-                            for (int v = 0; v < CF / E; ++v) {
-                                float f[E];
-                                FeatVec<FT>::lds(&G.row[buf][j][v * E], f);
+                for (int i = 0; i < H; ++i) {
+                    sel[i] = false;
+                    wsel[i] = 0.0f;
+                    Hit h;
+                    if (H == 2 && i == 1 && !((lower >> j) & 1u)) continue;
+                    if (pos < nstop[i] &&
+                        eval_splat<VAR>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf + (float)(4 * i), P.alpha_min, cam.near_plane, h,
+                                        P.lowpass)) {
+                        contrib = true;
+                        const float alpha = fminf(h.alpha_raw, P.alpha_max);
+                        const float Tj = T[i] * rcp_approx(1.0f - alpha);
+                        const float w = alpha * Tj;
+                        float s = oc.y * gr[i] + oc.z * gg[i] + oc.w * gb[i];
+                        if (pos == next_pos[i]) {
+                            if constexpr (CF > 0) {
+                                float2 d0 = make_float2(0.0f, 0.0f), d1 = d0;
 #pragma unroll
-                                for (int e = 0; e < E / 2; e += 2) {
-                                    d0 = __ffma2_rn(make_float2(f[2 * e], f[2 * e + 1]), dfr[v * (E / 2) + e], d0);
-                                    d1 = __ffma2_rn(make_float2(f[2 * e + 2], f[2 * e + 3]), dfr[v * (E / 2) + e + 1], d1);
+                                for (int v = 0; v < CF / E; ++v) {
+                                    float f[E];
+                                    FeatVec<FT>::lds(&G.row[buf][j][v * E], f);
+#pragma unroll
+                                    for (int e = 0; e < E / 2; e += 2) {
+                                        d0 = __ffma2_rn(make_float2(f[2 * e], f[2 * e + 1]), dfr[i][v * (E / 2) + e], d0);
+                                        d1 = __ffma2_rn(make_float2(f[2 * e + 2], f[2 * e + 3]), dfr[i][v * (E / 2) + e + 1], d1);
+                                    }
+                                }
+                                s += (d0.x + d0.y) + (d1.x + d1.y);
+                                sel[i] = true;
+                                wsel[i] = next_dot[i];
+                            } else {
+                                s += VAR ? fmaf(next_dot[i], rn_a[i], rn_b[i]) : next_dot[i];
+                            }
+                            const int k = --kk[i];
+                            const int64_t at = (pix0 + (int64_t)(4 * i) * cam.W) * K + k;
+                            next_pos[i] = k >= 0 ? a.saved_pos[at] : -1;
+                            next_dot[i] = k >= 0 ? (CF == 0 ? a.dots : a.saved_w)[at] : 0.0f;
+                        }
+                        const float dal = Tj * (s - Sh[i]);
+                        Sh[i] = fmaf(alpha, s - Sh[i], Sh[i]);  // a s + (1 - a) S
+                        g[10] = i ? fmaf(w, gr[i], g[10]) : w * gr[i];
+                        g[11] = i ? fmaf(w, gg[i], g[11]) : w * gg[i];
+                        g[12] = i ? fmaf(w, gb[i], g[12]) : w * gb[i];
+                        if (h.alpha_raw < P.alpha_max) {
+                            g[9] = i ? fmaf(dal, h.G, g[9]) : dal * h.G;
+                            const float drho = -0.5f * alpha * dal;
+                            if (VAR && h.scr) {  // low-pass screen term: rho = 2 |x - c|^2, d rho / d c = -4 (X, Y)
+                                g[VAR ? 13 : 0] += -4.0f * h.X * drho;
+                                g[VAR ? 14 : 0] += -4.0f * h.Y * drho;
+                            } else {
+                                const float du = 2.0f * h.u * drho, dv = 2.0f * h.v * drho;
+                                const float gc0 = du * h.inv, gc1 = dv * h.inv, gc2 = -(du * h.u + dv * h.v) * h.inv;
+                                if (i == 0) {
+                                    g[0] = gc0 * h.X; g[1] = gc0 * h.Y; g[2] = gc0;
+                                    g[3] = gc1 * h.X; g[4] = gc1 * h.Y; g[5] = gc1;
+                                    g[6] = gc2 * h.X; g[7] = gc2 * h.Y; g[8] = gc2;
+                                } else {
+                                    g[0] = fmaf(gc0, h.X, g[0]); g[1] = fmaf(gc0, h.Y, g[1]); g[2] += gc0;
+                                    g[3] = fmaf(gc1, h.X, g[3]); g[4] = fmaf(gc1, h.Y, g[4]); g[5] += gc1;
+                                    g[6] = fmaf(gc2, h.X, g[6]); g[7] = fmaf(gc2, h.Y, g[7]); g[8] += gc2;
                                 }
                             }
-                            s += (d0.x + d0.y) + (d1.x + d1.y);
-                            sel = true;
-                            wsel = next_dot;
-                        } else {
-                            s += VAR ? fmaf(next_dot, rn_a, rn_b) : next_dot;
                         }
-                        --kk;
-                        next_pos = kk >= 0 ? a.saved_pos[pix * K + kk] : -1;
-                        next_dot = kk >= 0 ? (CF == 0 ? a.dots : a.saved_w)[pix * K + kk] : 0.0f;
+                        T[i] = Tj;
                     }
-                    const float dal = Tj * (s - Sh);
-                    Sh = fmaf(alpha, s - Sh, Sh);  // a s + (1 - a) S
-                    g[10] = w * gr;
-                    g[11] = w * gg;
-                    g[12] = w * gb;
-                    if (h.alpha_raw < P.alpha_max) {
-                        g[9] = dal * h.G;
-                        const float drho = -0.5f * alpha * dal;
-                        if (VAR && h.scr) {  // low-pass screen term: rho = 2 |x - c|^2, d rho / d c = -4 (X, Y)
-                            g[VAR ? 13 : 0] = -4.0f * h.X * drho;
-                            g[VAR ? 14 : 0] = -4.0f * h.Y * drho;
-                        } else {
-                            const float du = 2.0f * h.u * drho, dv = 2.0f * h.v * drho;
-                            const float gc0 = du * h.inv, gc1 = dv * h.inv, gc2 = -(du * h.u + dv * h.v) * h.inv;
-                            g[0] = gc0 * h.X; g[1] = gc0 * h.Y; g[2] = gc0;
-                            g[3] = gc1 * h.X; g[4] = gc1 * h.Y; g[5] = gc1;
-                            g[6] = gc2 * h.X; g[7] = gc2 * h.Y; g[8] = gc2;
-                        }
-                    }
-                    T = Tj;
                 }
                 if (__any_sync(ALL, contrib)) {
                     if constexpr (VAR) reduce_scatter<16>(g);  // lane l holds value l >> 1
@@ -663,12 +699,16 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
                     if ((lane & 1) == 0 && (lane >> 1) < (VAR ? 15 : 13) && in_bounds(a.st, SITE_SLOT, slot, P.N))
                         atomicAdd(grows + (int64_t)slot * GRAD_STRIDE + (lane >> 1), g[0]);
                     if constexpr (CF > 0) {
-                        if (__any_sync(ALL, sel)) {
+                        if (__any_sync(ALL, sel[0] || sel[H - 1])) {
                             float gf[CF];
 #pragma unroll
                             for (int c = 0; c < CF / 2; ++c) {
-                                gf[2 * c] = sel ? wsel * dfr[c].x : 0.0f;  // (dL/dF may be infinite where not selected)
-                                gf[2 * c + 1] = sel ? wsel * dfr[c].y : 0.0f;
+                                gf[2 * c] = sel[0] ? wsel[0] * dfr[0][c].x : 0.0f;  // (dL/dF may be infinite where not selected)
+                                gf[2 * c + 1] = sel[0] ? wsel[0] * dfr[0][c].y : 0.0f;
+                                if (H == 2 && sel[H - 1]) {
+                                    gf[2 * c] = fmaf(wsel[H - 1], dfr[H - 1][c].x, gf[2 * c]);
+                                    gf[2 * c + 1] = fmaf(wsel[H - 1], dfr[H - 1][c].y, gf[2 * c + 1]);
+                                }
                             }
                             reduce_scatter<CF>(gf);  // lane l holds channel l (CF = 32) or l >> 1
                             const int c = CF == 32 ? lane : lane >> 1;
@@ -679,6 +719,7 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT>(),
                 }
             }
             word = next;
+            lower = lower_next;
             __syncwarp();  // every lane has read this half before the next copies into it
         }
         cp_async_wait_all();
@@ -1314,12 +1355,13 @@ cudaError_t launch_geo_full(const Cams& cams, const RParams& P, const BwdArgs& a
 //   183 / 199; of 32: 128 x 128 443 / 334).
 // Neither with a renormalised selection, which needs every dot before the first, nor with
 // the other variants.
-enum FeatPath { FEAT_KERNEL, FEAT_REPLAY, FEAT_PRODUCTS };
+enum FeatPath { FEAT_KERNEL, FEAT_REPLAY, FEAT_REPLAY_TWO, FEAT_PRODUCTS };
 FeatPath feat_path(const Cams& cams, const RParams& P, int num_sms) {
     if (P.K == 0 || P.renorm || P.color_sh || P.lowpass) return FEAT_KERNEL;
     const bool half = P.feat_dtype == FSS_BF16;
-    if (P.K > 8 && P.C <= (half ? 32 : 16)) return FEAT_REPLAY;
     const int64_t blocks = (int64_t)cams.total_tiles * (P.ts * P.ts / 32);
+    if (P.K > 8 && P.C <= 16) return blocks >= (int64_t)num_sms * 48 ? FEAT_REPLAY_TWO : FEAT_REPLAY;
+    if (P.K > 8 && P.C <= 32 && half) return FEAT_REPLAY;
     if (blocks >= (int64_t)num_sms * (P.ts == 8 ? 8 : P.ts == 16 ? (half ? 4 : 2) : 0) &&
         (half ? P.C > 32 && P.C <= 64 && P.C * P.K >= 1152
               : P.C > 16 && P.C <= 128 && P.C * P.K >= (P.C <= 64 ? 288 : 1200) && (P.C > 32 || P.K > 8)))
@@ -1329,8 +1371,8 @@ FeatPath feat_path(const Cams& cams, const RParams& P, int num_sms) {
 
 template <int TS, typename FT>
 cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a, FeatPath feat, cudaStream_t s) {
-    auto go = [&](auto kern, int nt) {
-        int64_t units = (int64_t)cams.total_tiles * (TS * TS / nt);
+    auto go = [&](auto kern, int nt, int h = 1) {
+        int64_t units = (int64_t)cams.total_tiles * (TS * TS / h / nt);
         if (a.persistent) {
             int wave = (int)std::min<int64_t>(units, INT_MAX);
             const cudaError_t e = persistent_grid((const void*)kern, nt, 0, wave);
@@ -1349,11 +1391,13 @@ cudaError_t launch_geo_topk(const Cams& cams, const RParams& P, const BwdArgs& a
         if (P.C <= 64) return launch_geo_full<TS, 64, FT, false, true>(cams, P, a, s);
         if constexpr (sizeof(FT) == 4) return launch_geo_full<TS, 128, FT, false, true>(cams, P, a, s);
     }
-    if (feat == FEAT_REPLAY)
-        return P.C <= 16 ? go(k_bwd_geo_topk<TS, false, 16, FT>, geo_threads<TS, 16, FT>())
-                         : go(k_bwd_geo_topk<TS, false, 32, FT>, geo_threads<TS, 32, FT>());
-    return P.renorm || P.color_sh || P.lowpass ? go(k_bwd_geo_topk<TS, true>, geo_threads<TS, 0, float>())
-                                               : go(k_bwd_geo_topk<TS, false>, geo_threads<TS, 0, float>());
+    if (feat != FEAT_KERNEL) {
+        if (feat == FEAT_REPLAY_TWO) return go(k_bwd_geo_topk<TS, false, 16, FT, 2>, geo_threads<TS, 16, FT, 2>(), 2);
+        return P.C <= 16 ? go(k_bwd_geo_topk<TS, false, 16, FT>, geo_threads<TS, 16, FT, 1>())
+                         : go(k_bwd_geo_topk<TS, false, 32, FT>, geo_threads<TS, 32, FT, 1>());
+    }
+    if (P.renorm || P.color_sh || P.lowpass) return go(k_bwd_geo_topk<TS, true>, geo_threads<TS, 0, float, 1>());
+    return go(k_bwd_geo_topk<TS, false>, geo_threads<TS, 0, float, 1>());
 }
 
 template <int TS, typename FT>

@@ -29,6 +29,18 @@ def test_feature_gradients_in_the_replay(C, dtype, K, ts):
     _check(sc, cam, K, dtype, tile_size=ts, seed=C + K)
 
 
+@pytest.mark.parametrize("C,dtype,ts,W,H", [(12, torch.float32, 16, 605, 413), (16, torch.bfloat16, 8, 604, 415),
+                                           (16, torch.float32, 32, 640, 410)])
+def test_two_blocks_per_warp(C, dtype, ts, W, H):
+    """Images large enough for the warps with two blocks; ragged below and to the right."""
+    sc, cam = scenes.tiny_scene(seed=9, n=600, C=C)
+    sc.opacities *= np.float32(0.4)
+    s = W / cam.width
+    big = scenes.Camera(cam.fx * s, cam.fy * s, W / 2, H / 2, W, H, cam.viewmat)
+    assert -(-W // ts) * -(-H // ts) * (ts * ts // 32) >= 48 * torch.cuda.get_device_properties(0).multi_processor_count
+    _check(sc, big, 12, dtype, tile_size=ts, seed=C)
+
+
 @pytest.mark.parametrize("C", [16, 32, 64])
 def test_an_infinite_gradient_stays_with_its_surfels(C):
     sc, cam = scenes.tiny_scene(seed=5, n=1200, C=C)
