@@ -1427,15 +1427,19 @@ cudaError_t launch_all(const Cams& cams, const RParams& P, const BwdArgs& a, con
     }
     // Once the feature gradients are complete their output pass (memory bound)
     // runs in a second stream, launched eagerly, beside the geometry replay
-    // (issue bound; 10 us less per 500k-surfel frame) or, where the replay took
-    // them, beside the projection, and joins before the call returns.  A graph
+    // (issue bound; 10 us less per 500k-surfel frame of 64 channels) or, where the
+    // replay took them, beside the projection (4 us), and joins before the call
+    // returns.  Below 48 MB of rows it costs the host more than it saves (four
+    // calls, 10 us: autograd steps that the host bounds, 100k surfels 407 -> 399
+    // us without it, 300k 421 -> 413; 1296 x 968 with 32 MB 1032 -> 1035).  A graph
     // being captured keeps one stream: replayed, the branch measured 3 us slower
     // than the chain.
+    constexpr int64_t FORK_BYTES = 48 << 20;
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return e;
-    const bool fork = a.g_feat && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
+    const bool fork = a.g_feat && P.N * P.C * (int64_t)sizeof(FT) >= FORK_BYTES && cap == cudaStreamCaptureStatusNone && !kernel_marks_armed() &&
                       side_stream(s, side, ev_fork, ev_join);
     bool forked = false;
     auto rows_beside = [&]() {
