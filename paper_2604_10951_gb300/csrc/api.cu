@@ -146,15 +146,11 @@ Layout make_layout(const RParams& P, const Cams& cams) {
     sz[REG_COLOR] = P.color_sh ? ni * 12 : 0;
     sz[REG_ORDER] = (size_t)cams.total_tiles * 4;
     size_t off = 0;
-    auto place = [&](int r) {
+    for (int r = 0; r < REG_COUNT_ALL; ++r) {
         L.off[r] = off;
         L.size[r] = sz[r];
         off += align256(sz[r]) + GUARD_BYTES;  // check build: the region's canary follows it
-    };
-    place(REG_STATUS);
-    place(REG_TILECNT);  // behind the status block: cleared with it by one memset
-    for (int r = 0; r < REG_COUNT_ALL; ++r)
-        if (r != REG_STATUS && r != REG_TILECNT) place(r);
+    }
     L.off[REG_COUNTERS] = L.off[REG_STATUS] + STATUS_CLEAR_OFF;
     L.size[REG_COUNTERS] = sizeof(((Status*)0)->counters);
     L.total = off;
@@ -382,18 +378,14 @@ fss_status fss_project_bin(const fss_params* params, const fss_camera* cams, int
         return fail(FSS_ERR_INVALID_ARG, "quats must be 16-byte and scales 8-byte aligned");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e;
-    // clear the per-frame part of the status block and the tile counts (adjacent
-    // regions) and, for several views, the gradient slots (with one view the
-    // projection writes every slot)
-    const size_t clear = ctx.L.off[REG_STATUS] + STATUS_CLEAR_OFF;
-    e = cudaMemsetAsync(ctx.ws + clear, 0, ctx.L.off[REG_TILECNT] + ctx.L.size[REG_TILECNT] - clear, st);
-    if (e != cudaSuccess) return cuda_fail(e, "memset status and tile counts");
-    if (N > 0 && ctx.cams.n > 1) {
-        e = cudaMemsetAsync(ctx.ws + ctx.L.off[REG_SLOT], 0xff, (size_t)N * 4, st);
-        if (e != cudaSuccess) return cuda_fail(e, "memset slots");
-    }
-    if ((e = arm_guards(ctx, st)) != cudaSuccess) return cuda_fail(e, "memset canaries");
     const int sms = num_sms_current();
+    // the per-frame part of the status block, the tile counts and, for several views,
+    // the gradient slots (with one view the projection writes every slot)
+    e = launch_bin_clear(ctx.at<uint32_t>(REG_STATUS) + STATUS_CLEAR_OFF / 4, (sizeof(Status) - STATUS_CLEAR_OFF) / 4,
+                         ctx.at<uint4>(REG_TILECNT), (int64_t)ctx.L.size[REG_TILECNT] / 16,
+                         ctx.at<int32_t>(REG_SLOT), ctx.cams.n > 1 ? N : 0, sms, st);
+    if (e != cudaSuccess) return cuda_fail(e, "k_bin_clear");
+    if ((e = arm_guards(ctx, st)) != cudaSuccess) return cuda_fail(e, "memset canaries");
     Status* stp = ctx.at<Status>(REG_STATUS);
     e = launch_project(ctx.cams, ctx.P, means, scales, quats, opac, ctx.at<float4>(REG_REC), ctx.at<BinRec>(REG_BINREC),
                        ctx.at<uint32_t>(REG_COUNT), ctx.at<uint32_t>(REG_TILECNT), ctx.at<uint32_t>(REG_VIS),

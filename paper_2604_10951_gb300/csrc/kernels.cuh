@@ -26,6 +26,8 @@ bool kernel_marks_armed();
 bool side_stream(cudaStream_t s, cudaStream_t& side, cudaEvent_t& fork, cudaEvent_t& join);
 
 // projection and tile counts (k_project)
+cudaError_t launch_bin_clear(uint32_t* status, int status_words, uint4* tile_cnt, int64_t tile_vecs, int32_t* slot,
+                             int64_t slots, int num_sms, cudaStream_t stream);
 cudaError_t launch_project(const Cams& cams, const RParams& P, const float* means, const float* scales, const float* quats,
                            const float* opac, float4* rec, BinRec* binrec, uint32_t* count, uint32_t* tile_cnt,
                            uint32_t* vis_list, uint32_t* wide_list, uint32_t* unb_list, int32_t* splat_slot,

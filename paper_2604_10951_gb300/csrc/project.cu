@@ -775,6 +775,27 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     }  // survivors
 }
 
+// Before binning: zeros for the status block's per-frame words and the tile counts
+// (16-byte vectors), -1 for the gradient slots (none with one view).  One launch of a
+// few microseconds where each of the regions took a memset; not one of the kernels that the
+// measurement hook counts.
+__global__ void __launch_bounds__(256) k_bin_clear(uint32_t* status, int status_words, uint4* tile_cnt, int64_t tile_vecs,
+                                                   int32_t* slot, int64_t slots) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < status_words; i += n) status[i] = 0u;
+    for (int64_t i = i0; i < tile_vecs; i += n) tile_cnt[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t i = i0; i < slots / 4; i += n) reinterpret_cast<int4*>(slot)[i] = make_int4(-1, -1, -1, -1);
+    for (int64_t i = slots / 4 * 4 + i0; i < slots; i += n) slot[i] = -1;
+}
+
+cudaError_t launch_bin_clear(uint32_t* status, int status_words, uint4* tile_cnt, int64_t tile_vecs, int32_t* slot,
+                             int64_t slots, int num_sms, cudaStream_t stream) {
+    const int64_t work = std::max<int64_t>(status_words, std::max<int64_t>(tile_vecs, slots / 4));
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 4 * (int64_t)num_sms));
+    k_bin_clear<<<blocks, 256, 0, stream>>>(status, status_words, tile_cnt, tile_vecs, slot, slots);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_project(const Cams& cams, const RParams& P, const float* means, const float* scales, const float* quats,
                            const float* opac, float4* rec, BinRec* binrec, uint32_t* count, uint32_t* tile_cnt,
                            uint32_t* vis_list, uint32_t* wide_list, uint32_t* unb_list, int32_t* splat_slot,
