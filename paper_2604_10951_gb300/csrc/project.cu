@@ -5,11 +5,13 @@
 //             screen conic, SnugBox pixel range; appends visible items to a
 //             compact list (unbounded conics to a per-view list instead).
 //             Also counts each item's tiles (AccuTile per-row or per-column
-//             intervals) into per-tile counters.
+//             intervals) into per-tile counters; a narrow item's pairs (tile,
+//             place in the tile, item) go into a buffer in the same pass.
 // k_emit      computes the double-float render records; one of its CTAs
 //             scans the per-tile counts (tile ranges, total pairs, capacity,
 //             the heavy-first tile order) while the others build records;
-//             then writes each item into a slot of each of its tiles (slot
+//             then stores the buffered pairs at their tile's cursor + place and
+//             writes each wide item into a slot of each of its tiles (slot
 //             order is arbitrary; the per-tile sort restores a total order).
 //
 // Every tile decision is taken in binary32 with the fixed operation order
