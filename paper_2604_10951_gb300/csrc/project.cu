@@ -23,7 +23,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <type_traits>
 
 namespace fss {
 
@@ -397,7 +396,7 @@ __device__ __forceinline__ bool surely_culled(const CamDev& cam, const RParams& 
 constexpr int PROJ_THREADS = 256;
 
 // ---------------------------------------------------------------------------
-// k_project: (view, surfel) items, PER * 256 per CTA
+// k_project: (view, surfel) items, ROUNDS * PER * 256 per CTA
 //
 // Stage A drops the items that the cheap superset of the culls is sure about,
 // one thread per item, and queues the rest in shared memory; stage B runs the
@@ -415,7 +414,12 @@ constexpr int PROJ_THREADS = 256;
 // PER = 4 packs stage B well where most items are culled; PER = 1 spreads few
 // items over the SMs: below 1024 items per SM (1,000 surfels in a 128 x 128
 // frame: 66 -> 41 us for the whole forward, with PER = 4 62; 150k in a room 73
-// -> 69, 71; 300k 87 -> 89, 85).  Stage A is bound by the latency of its loads;
+// -> 69, 71; 300k 87 -> 89, 85).  From 4096 and 8192 items per SM a CTA runs stage A
+// two and three times before its stage B: the survivors of 1024 items (a twentieth)
+// leave most of its warps without a stage B, whose chain the CTA waits for, and the CTAs
+// are one wave again (4 an SM).  Whole forwards, one / two / three rounds: 800k items
+// 116 / 110 / 113 us, 1M 121 / 115 / 122, 1.5M 253 / 254 / 246 (four: 255), 3M in five
+// views 295 / 288 / 286 (four: 296), 12M in twelve 1397 / 1331 / 1316.  Stage A is bound by the latency of its loads;
 // with the exact culls in it (a logarithm, a square root and four divisions per
 // item) 1.5M items took 50 us where this takes 42, and 12M items 279 / 220.
 // ---------------------------------------------------------------------------
@@ -426,8 +430,9 @@ constexpr int PROJ_THREADS = 256;
 constexpr uint32_t WIDE_TILES = 256;
 constexpr int PAIR_BATCH = 8;  // tile counters added to at once by a lane (4: 411 us)
 constexpr int64_t PROJ_SPREAD = 1024;  // items per SM below which a CTA takes 256 of them
+constexpr int64_t PROJ_TWO = 4096, PROJ_THREE = 8192;  // ... from which it takes twice, three times 1024
 
-template <int PER>
+template <int PER, int ROUNDS>
 __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_constant__ Cams cams, const __grid_constant__ RParams P,
                                                  const float* __restrict__ means, const float* __restrict__ scales,
                                                  const float* __restrict__ quats, const float* __restrict__ opac,
@@ -437,7 +442,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
                                                  uint32_t* __restrict__ unb_list, int32_t* __restrict__ splat_slot,
                                                  int32_t* __restrict__ slot_surf, uint32_t* __restrict__ pairs,
                                                  Status* __restrict__ st, float rmax, float mmax) {
-    constexpr int PROJ_ITEMS = PER * PROJ_THREADS;
+    constexpr int PROJ_ITEMS = ROUNDS * PER * PROJ_THREADS;
     __shared__ uint32_t s_q[PROJ_ITEMS];
     __shared__ int s_nq;
     __shared__ BinRec s_br[PROJ_THREADS];
@@ -457,11 +462,13 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     // stage A: the superset of the culls for PROJ_ITEMS items (each thread's items
     // loaded together first); the rest queued in shared memory
     const int64_t base = (int64_t)blockIdx.x * PROJ_ITEMS;
+#pragma unroll 1
+    for (int k0 = threadIdx.x; k0 < PROJ_ITEMS; k0 += PER * PROJ_THREADS) {
     CullIn in[PER];
     int vw[PER];
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-        const int64_t it = base + threadIdx.x + i * PROJ_THREADS;
+        const int64_t it = base + k0 + i * PROJ_THREADS;
         vw[i] = 0;
         if (it < P.n_items) {
             vw[i] = view_of_item(it, P.N);
@@ -470,7 +477,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-        const int k = threadIdx.x + i * PROJ_THREADS;
+        const int k = k0 + i * PROJ_THREADS;
         const int64_t it = base + k;
         const bool keep = it < P.n_items && !surely_culled(cams.c[vw[i]], P, in[i], rmax, mmax);
         if (one_view && !keep && it < P.n_items) splat_slot[it] = -1;
@@ -479,6 +486,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, 4) k_project(const __grid_consta
         if (lane == 0 && m) b = atomicAdd(&s_nq, __popc(m));
         b = __shfl_sync(0xffffffffu, b, 0);
         if (keep) s_q[b + __popc(m & ((1u << lane) - 1u))] = (uint32_t)k;
+    }
     }
     __syncthreads();
     const int nq = s_nq;
@@ -806,15 +814,17 @@ cudaError_t launch_project(const Cams& cams, const RParams& P, const float* mean
     const double k2 = 2.0 * std::log(1.0 / (double)P.alpha_min) * 1.0009765625;
     const float rmax = (float)(std::sqrt(std::max(k2, 0.0)) * 1.0015);
     const float mmax = (float)(1.0 + (P.lowpass ? std::sqrt(std::max(k2, 0.0) * 0.5) * 1.0015 : 0.0));
-    auto go = [&](auto per) {
-        constexpr int PER = decltype(per)::value;
-        const int64_t blocks = std::max<int64_t>(1, (P.n_items + PER * PROJ_THREADS - 1) / (PER * PROJ_THREADS));
-        k_project<PER><<<(unsigned)blocks, PROJ_THREADS, 0, stream>>>(cams, P, means, scales, quats, opac, rec, binrec,
-                                                                    count, tile_cnt, vis_list, wide_list, unb_list,
-                                                                    splat_slot, slot_surf, pairs, st, rmax, mmax);
+    auto go = [&](auto kern, int64_t items) {
+        const int64_t blocks = std::max<int64_t>(1, (P.n_items + items - 1) / items);
+        kern<<<(unsigned)blocks, PROJ_THREADS, 0, stream>>>(cams, P, means, scales, quats, opac, rec, binrec, count, tile_cnt,
+                                                            vis_list, wide_list, unb_list, splat_slot, slot_surf, pairs, st,
+                                                            rmax, mmax);
         return cudaGetLastError();
     };
-    return P.n_items < PROJ_SPREAD * num_sms ? go(std::integral_constant<int, 1>{}) : go(std::integral_constant<int, 4>{});
+    if (P.n_items < PROJ_SPREAD * num_sms) return go(k_project<1, 1>, PROJ_THREADS);
+    if (P.n_items < PROJ_TWO * num_sms) return go(k_project<4, 1>, 4 * PROJ_THREADS);
+    if (P.n_items < PROJ_THREE * num_sms) return go(k_project<4, 2>, 8 * PROJ_THREADS);
+    return go(k_project<4, 3>, 12 * PROJ_THREADS);
 }
 
 // ---------------------------------------------------------------------------

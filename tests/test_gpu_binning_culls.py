@@ -3,7 +3,8 @@ lists bit-exact against the oracle for surfels crowded at the frustum's edges,
 of all sizes, nearly transparent and opaque, also with opacities above 1 (which
 it must leave to the exact test), for off-centre and telephoto cameras, with
 and without the low-pass filter, on both sides of its two launch shapes
-(few items: 256 per CTA; many: 1024).
+(few items: 256 per CTA; many: 1024), and with the two and three times 1024
+of still more.
 """
 import numpy as np
 import pytest
@@ -45,5 +46,14 @@ def test_edge_surfels_many_items():
     cams = [ident_cam(W=48, H=48, f=50.0), ident_cam(W=64, H=32, f=40.0, cx=-20.0)]
     sc = _edge_scene(90_000, cams[0], seed=3)
     sc.scales *= np.float32(0.2)
+    run = GpuRun(sc, cams, K=4, render=False, cap=1 << 23)
+    _check_lists(run, sc, cams, 16, "accu")
+
+
+@pytest.mark.parametrize("views", [8, 15])  # 672k and 1.26M items: two and three rounds per CTA
+def test_edge_surfels_many_views(views):
+    cams = [ident_cam(W=40 + v, H=30, f=40.0 + 2 * v, cx=20.0 * (v % 3), cy=15.0) for v in range(views)]
+    sc = _edge_scene(84_001, cams[0], seed=4)
+    sc.scales *= np.float32(0.05)
     run = GpuRun(sc, cams, K=4, render=False, cap=1 << 23)
     _check_lists(run, sc, cams, 16, "accu")
