@@ -48,11 +48,11 @@ namespace fss {
 // Top-K kernel
 // ---------------------------------------------------------------------------
 // The K-set of a pixel lives in registers as an array sorted by decreasing
-// weight.  A new weight x takes its place in one step per slot, all slots at
-// once from the last up: slot k becomes the middle one of (slot k - 1, x, slot
-// k), i.e. max(slot k, min(slot k - 1, x)), and its position follows the two
-// strict comparisons, so between equal weights the earlier surfel stays in
-// front and the later one is the first to fall off the end.  For K < KCAP
+// weight.  A new weight x takes its place and each one behind it moves on by a slot:
+// the weight carried into slot k is min(slot k - 1, x), known for all slots at once,
+// and it stays there if it exceeds the slot's, so only the positions pass from slot
+// to slot.  An equal weight in a slot stays and the carried one goes on behind it: a new
+// weight never displaces an equal one.  For K < KCAP
 // the first KCAP - K slots hold +inf and never move, so the K-th largest
 // weight is always slot KCAP - 1.  With the first-K selection the K slots
 // after the padding take the first K contributors in order.
@@ -217,12 +217,17 @@ __global__ void __launch_bounds__(topk_threads<TS, SORT>(), (KCAP <= 8 ? 1024 : 
                         ++n_sel;
                     }
                 } else if (w > hw[KCAP - 1]) {
+                    float in[KCAP];
+                    int cp = b0 + j;  // the position carried into slot k, with weight min(slot k - 1, w)
 #pragma unroll
-                    for (int k = KCAP - 1; k >= 0; --k) {
-                        const bool here = w > hw[k];  // w belongs in this slot or in front of it
-                        const bool above = k > 0 && w > hw[k > 0 ? k - 1 : 0];
-                        hp[k] = here ? (above ? hp[k > 0 ? k - 1 : 0] : b0 + j) : hp[k];
-                        hw[k] = k > 0 ? fmaxf(hw[k], fminf(hw[k > 0 ? k - 1 : 0], w)) : fmaxf(hw[0], w);
+                    for (int k = KCAP - 1; k >= 0; --k) in[k] = k > 0 ? fminf(hw[k > 0 ? k - 1 : 0], w) : w;
+#pragma unroll
+                    for (int k = 0; k < KCAP; ++k) {
+                        const bool gt = in[k] > hw[k];
+                        const int np = gt ? cp : hp[k];
+                        cp = gt ? hp[k] : cp;
+                        hp[k] = np;
+                        hw[k] = fmaxf(hw[k], in[k]);
                     }
                 }
                 T = Tn;

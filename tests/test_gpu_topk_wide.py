@@ -40,7 +40,7 @@ def test_more_contributors_than_slots(K, ts, stop, kw):
     _compare(run.view(0), ref, S, 1e-4, K)
 
 
-@pytest.mark.parametrize("K", [9, 24, 32])
+@pytest.mark.parametrize("K", [17, 24, 32])
 def test_equal_weights_keep_the_earlier_surfel(K):
     """Surfels facing the camera, all centred on one pixel's ray, so that alpha is the
     opacity itself there: the weights are what the binary32 recurrence T (1 - alpha)
@@ -70,6 +70,42 @@ def test_equal_weights_keep_the_earlier_surfel(K):
             equal += sum(s[0] == low for s in sel) > 1
             sel.remove(max(s for s in sel if s[0] == low))
             sel.append((w, i))
+    assert equal > 0
+    v = run.view(0)
+    np.testing.assert_array_equal(v["ids"][16, 16], sorted(i for _, i in sel))
+    np.testing.assert_array_equal(v["w"][16, 16], [w for w, _ in sorted(sel, key=lambda s: s[1])])
+
+
+@pytest.mark.parametrize("K", [4, 8, 9, 16])
+def test_equal_weights_as_an_insertion_chain(K):
+    """Surfels facing the camera, all centred on one pixel's ray, so that alpha is the
+    opacity itself there: the weights are what the binary32 recurrence T (1 - alpha)
+    gives, with many equal ones, and later ones that push one of the equals out: with the set in
+    registers (K <= 16) the one that an insertion chain (each larger weight moves the ones behind it on, an equal one
+    stays in its slot) carries off the end."""
+    n = 3 * K
+    c = np.float32(1.0 / 128.0)
+    o, T = [], np.float32(1.0)
+    for i in range(n):
+        a = np.float32(c / T) if i % 7 != 6 else np.float32(2 * c / T)
+        o.append(a)
+        T = np.float32(T * np.float32(np.float32(1.0) - a))
+    means = np.stack([np.zeros(n), np.zeros(n), 2.0 + 0.01 * np.arange(n)], 1)
+    quats = np.tile([1.0, 0.0, 0.0, 0.0], (n, 1))
+    sc = make_scene(means, np.full((n, 2), 0.2), quats, np.array(o), C=8)
+    cam = ident_cam(W=32, H=32, f=32.0)
+    cam.cx = cam.cy = 16.5
+    run = GpuRun(sc, [cam], K=K)
+    sel, T, equal = [], np.float32(1.0), 0
+    for i, a in enumerate(np.asarray(sc.opacities, np.float32)):
+        w = np.float32(a * T)
+        T = np.float32(T * np.float32(np.float32(1.0) - a))
+        if len(sel) == K and w > sel[-1][0]:
+            equal += sel[-1][0] == sel[-2][0]
+        x, sel = (w, i), sel + [(np.float32(-1.0), -1)] * (len(sel) < K)
+        for k in range(len(sel)):
+            if x[0] > sel[k][0]:
+                x, sel[k] = sel[k], x
     assert equal > 0
     v = run.view(0)
     np.testing.assert_array_equal(v["ids"][16, 16], sorted(i for _, i in sel))
