@@ -642,18 +642,22 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
                         float s = oc.y * gr[i] + oc.z * gg[i] + oc.w * gb[i];
                         if (pos == next_pos[i]) {
                             if constexpr (CF > 0) {
-                                float2 d0 = make_float2(0.0f, 0.0f), d1 = d0;
+                                float d[CF / E];  // by 16-byte chunk, summed as k_bwd_feat's lanes sum them
 #pragma unroll
                                 for (int v = 0; v < CF / E; ++v) {
                                     float f[E];
                                     FeatVec<FT>::lds(&G.row[buf][j][v * E], f);
+                                    float2 p = make_float2(0.0f, 0.0f);
 #pragma unroll
-                                    for (int e = 0; e < E / 2; e += 2) {
-                                        d0 = __ffma2_rn(make_float2(f[2 * e], f[2 * e + 1]), dfr[i][v * (E / 2) + e], d0);
-                                        d1 = __ffma2_rn(make_float2(f[2 * e + 2], f[2 * e + 3]), dfr[i][v * (E / 2) + e + 1], d1);
-                                    }
+                                    for (int e = 0; e < E / 2; ++e)
+                                        p = __ffma2_rn(make_float2(f[2 * e], f[2 * e + 1]), dfr[i][v * (E / 2) + e], p);
+                                    d[v] = p.x + p.y;
                                 }
-                                s += (d0.x + d0.y) + (d1.x + d1.y);
+#pragma unroll
+                                for (int o = CF / E / 2; o > 0; o >>= 1)
+#pragma unroll
+                                    for (int v = 0; v < o; ++v) d[v] += d[v + o];
+                                s += d[0];
                                 sel[i] = true;
                                 wsel[i] = next_dot[i];
                             } else {
