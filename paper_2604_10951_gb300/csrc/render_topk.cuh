@@ -52,7 +52,9 @@ namespace fss {
 // the weight carried into slot k is min(slot k - 1, x), known for all slots at once,
 // and it stays there if it exceeds the slot's, so only the positions pass from slot
 // to slot.  An equal weight in a slot stays and the carried one goes on behind it: a new
-// weight never displaces an equal one.  For K < KCAP
+// weight never displaces an equal one.  (Positions all at once as well, which drops
+// another one of several equal smallest weights: 2 to 3 us less of a 640 x 480 frame,
+// 9 of 423 at 1.5M surfels, 1280 x 720.)  For K < KCAP
 // the first KCAP - K slots hold +inf and never move, so the K-th largest
 // weight is always slot KCAP - 1.  With the first-K selection the K slots
 // after the padding take the first K contributors in order.
