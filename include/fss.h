@@ -179,10 +179,15 @@ fss_status fss_sort(const fss_params *params, const fss_camera *cams, int32_t n_
  * (u,v), alpha = min(alpha_max, o exp(-(u^2+v^2)/2)), skip if
  * alpha < alpha_min, stop by params->stop_rule, w = alpha T, T *= 1 - alpha.
  * K = 0: F = sum_i w_i c_i over all contributors.  K > 0: F = sum over the K
- * largest w_i (ties: earlier wins; FSS_SELECT_FRONT: over the first K
- * contributors), no renormalisation unless params->renorm (then divided by
- * the sum of the selected w_i; saved weights stay unnormalised).  FSS_STOP_EXACT_TOPK stops once no
- * later surfel can enter the set (TOPW: alpha_max T <= smallest selected
+ * largest w_i (FSS_SELECT_FRONT: over the first K contributors).  Exact ties
+ * for the last places, whatever the outputs asked for: a later surfel never
+ * displaces one of equal weight; a surfel of larger weight takes the place of
+ * the latest of the equal ones for K > 16, and for K <= 16 of the one that an
+ * insertion chain carries off the end (a larger weight moves the ones behind
+ * it on by a slot, an equal one keeps its slot).  No renormalisation unless
+ * params->renorm (then divided by the sum of the selected w_i; saved weights
+ * stay unnormalised).  FSS_STOP_EXACT_TOPK stops once no later surfel can
+ * enter the set (TOPW: alpha_max T <= smallest selected
  * weight; FRONT: K contributors found).
  * Device inputs: rgb [N,3] f32, feats [N,C] (feat_dtype).
  * Device outputs (any may be NULL except as noted; per view concatenated):

@@ -10,7 +10,7 @@
 //   at a time (stage_chunk: asynchronous copies into its own double buffer);
 //   every lane intersects its pixel ray with each staged surfel, composites
 //   colour and transmittance and keeps its K largest blending weights in
-//   registers (ties keep the earlier surfel).  The warp leaves the loop as
+//   registers (ties: see the K-set below).  The warp leaves the loop as
 //   soon as all its pixels have stopped.
 // Phase 2: the warp gathers only the K selected feature rows per pixel
 //   (16-byte loads: 8 bf16 or 4 f32 channels), weights them in FP32 and writes
@@ -52,7 +52,9 @@ namespace fss {
 // the weight carried into slot k is min(slot k - 1, x), known for all slots at once,
 // and it stays there if it exceeds the slot's, so only the positions pass from slot
 // to slot.  An equal weight in a slot stays and the carried one goes on behind it: a new
-// weight never displaces an equal one.  (Positions all at once as well, which drops
+// weight never displaces an equal one, and of several equal smallest ones the first in the
+// chain's order falls off, which need not be the latest (chain_leaver in render_topk_wide.cuh
+// follows this for the variants' sets of the same size).  (Positions all at once as well, which drops
 // another one of several equal smallest weights: 2 to 3 us less of a 640 x 480 frame,
 // 9 of 423 at 1.5M surfels, 1280 x 720.)  For K < KCAP
 // the first KCAP - K slots hold +inf and never move, so the K-th largest
@@ -464,7 +466,7 @@ cudaError_t launch_topk(const Cams& cams, const RParams& P, const FwdArgs& a, co
     // larger sets live in shared memory (render_topk_wide.cuh): those of more than
     // 16 entries, and more than 8 for the variants, which need the registers
     const bool plain = !aux && P.select != FSS_SELECT_FRONT;
-    if (P.K > (plain ? 16 : 8)) return launch_topk_wide<TS, FT>(cams, P, a, x, num_sms, s);
+    if (P.K > (plain ? CHAIN_K : 8)) return launch_topk_wide<TS, FT>(cams, P, a, x, num_sms, s);
     auto go = [&](auto kern, int kcap = 8) { return launch_tiles(kern, NT, smem(kcap), cams, P, a, x, num_sms, s, PARTS); };
     if (P.select == FSS_SELECT_FRONT)
         return aux ? go(k_render_topk<TS, 8, FT, true, true>) : go(k_render_topk<TS, 8, FT, true, false>);

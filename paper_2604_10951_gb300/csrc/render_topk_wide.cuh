@@ -42,6 +42,46 @@ inline __host__ __device__ size_t wide_warp_smem(int K, bool aux) {
     return 2 * sizeof(WarpStage) + (aux ? 32 * (16 + 8) : 0) + (size_t)K * 32 * 8 + (size_t)((K * 32 + 15) & ~15) + 128;
 }
 
+// Which of several equal smallest weights leaves.  Sets of up to CHAIN_K entries follow the
+// insertion chain of render_topk.cuh, which keeps those of the plain frames: the outputs
+// asked for must not change the selection.  Larger sets drop the entry at the latest position.
+//
+// In the chain an insertion turns every run of equal smaller weights by one (its first entry
+// goes behind its last: equal ones stay in their slots) and the last run loses its first.  So
+// a run's order when its first entry leaves follows from the set as it is then: taken by
+// position, an entry of the run joins it behind the others, a larger one turns it.  (Smaller ones have
+// left, and larger ones cannot have.)  From then on entries only leave it, first to last, and
+// none joins: a weight enters only above the smallest.  The order is formed once per run,
+// into s_ord (free until the traversal ends; `tied` holds the run's weight), and the first of
+// it that is still in the set leaves.  Ties are rare: none of this runs otherwise.
+constexpr int CHAIN_K = 16;  // the largest set of render_topk.cuh
+__device__ __forceinline__ int chain_leaver(const float* s_kw, const int32_t* s_kp, unsigned char* s_ord, int32_t* tied,
+                                            int K, float wmin) {
+    const int lane = threadIdx.x & 31;
+    if (*tied != __float_as_int(wmin)) {
+        *tied = __float_as_int(wmin);
+        unsigned long long run = 0ull;  // its slots, first in the low bits, 4 bits each
+        int n = 0;
+        for (int i = 0, last = -1; i < K; ++i) {  // the entries by position
+            int s = 0, at = INT_MAX;
+            for (int j = 0; j < K; ++j) {
+                const int p = s_kp[j * 32 + lane];
+                if (p > last && p < at) {
+                    at = p;
+                    s = j;
+                }
+            }
+            last = at;
+            if (s_kw[s * 32 + lane] == wmin) run |= (unsigned long long)s << (4 * n++);
+            else if (n > 1) run = (run >> 4) | ((run & 15ull) << (4 * (n - 1)));
+        }
+        for (int i = 0; i < K; ++i) s_ord[i * 32 + lane] = (unsigned char)((run >> (4 * i)) & 15ull);  // (zeros behind it)
+    }
+    int i = 0;  // (entries that have left hold larger weights now)
+    while (i < K - 1 && s_kw[s_ord[i * 32 + lane] * 32 + lane] != wmin) ++i;
+    return s_ord[i * 32 + lane];
+}
+
 // the minimum of group g takes w in (scalars: an indexed array would go to local memory)
 __device__ __forceinline__ void group_min(int g, float w, float& m0, float& m1, float& m2, float& m3) {
     m0 = g == 0 ? fminf(m0, w) : m0;
@@ -112,6 +152,7 @@ __global__ void __launch_bounds__(TS * TS < WIDE_THREADS ? TS * TS : WIDE_THREAD
         uint32_t rep = 0u;                                      // refilled slots
         float gm0 = INFINITY, gm1 = INFINITY, gm2 = INFINITY, gm3 = INFINITY;  // minima of the slot groups
         float wmin = -INFINITY;                                 // smallest selected weight once K are selected
+        if (AUX) s_n[lane] = -1;                                // until the outputs: chain_leaver's run (none yet: a NaN)
         uint32_t n_eval = 0, n_contrib = 0;
         float zs = 0.0f, zmed = 0.0f, nx = 0.0f, ny = 0.0f, nz = 0.0f;  // AUX sums
         bool med = false;
@@ -187,11 +228,15 @@ __global__ void __launch_bounds__(TS * TS < WIDE_THREADS ? TS * TS : WIDE_THREAD
                             gm3 = g == 3 ? gn : gm3;
                             s_kw[slot * 32 + lane] = w;
                             s_kp[slot * 32 + lane] = b0 + j;
-                        } else {  // equal weights: the one at the latest position leaves
-                            int pl = -1;
-                            for (int s = 0; s < K; ++s) {
-                                const int p = s_kp[s * 32 + lane];
-                                if (s_kw[s * 32 + lane] == wmin && p > pl) { pl = p; slot = s; }
+                        } else {  // equal weights (see chain_leaver)
+                            if (AUX && K <= CHAIN_K) {
+                                slot = chain_leaver(s_kw, s_kp, s_ord, s_n + lane, K, wmin);
+                            } else {
+                                int pl = -1;
+                                for (int s = 0; s < K; ++s) {
+                                    const int p = s_kp[s * 32 + lane];
+                                    if (s_kw[s * 32 + lane] == wmin && p > pl) { pl = p; slot = s; }
+                                }
                             }
                             s_kw[slot * 32 + lane] = w;
                             s_kp[slot * 32 + lane] = b0 + j;
