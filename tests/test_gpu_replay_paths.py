@@ -1,0 +1,68 @@
+"""The backward replays at the sizes where their dispatch takes them: products shared by
+a warp's lanes with tiles of 8 and 16, in both types, on an image with enough blocks an SM (ragged to the
+right and below); and the feature rows written in the second stream after the replay.
+Gradients against the oracle's FP64 analytic ones, tolerances as in test_gpu_feat_grad_shapes.py;
+the second stream against the same call captured on one stream, tolerance as in
+test_gpu_autograd_graph.py (BF16 storage is not used).
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_10951_gb300 import scenes
+from paper_2604_10951_gb300.raster import Frame, make_params
+from tests.gpu_util import dev
+from tests.test_gpu_feat_grad_shapes import _check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("C,dtype,K,ts", [
+    (64, torch.float32, 24, 8), (20, torch.float32, 16, 8), (64, torch.bfloat16, 24, 8), (40, torch.bfloat16, 32, 16),
+    (64, torch.bfloat16, 18, 16), (128, torch.float32, 16, 16), (68, torch.float32, 20, 8), (64, torch.float32, 8, 16)])
+def test_products_on_tiles_of_8_and_16(C, dtype, K, ts):
+    W, H = 321, 243
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert -(-W // ts) * -(-H // ts) * (ts * ts // 32) >= 8 * sms  # the most that any of these asks for
+    sc, cam = scenes.tiny_scene(seed=61 + C, n=800, C=C)
+    sc.opacities *= np.float32(0.3)
+    s = W / cam.width
+    _check(sc, scenes.Camera(cam.fx * s, cam.fy * s, W / 2, H / 2, W, H, cam.viewmat), K, dtype, tile_size=ts, seed=C + K)
+
+
+@pytest.mark.parametrize("N,C,K", [(200_000, 64, 0), (800_000, 16, 12), (400_000, 32, 10)])
+def test_feature_rows_in_the_second_stream_after_the_replay(N, C, K):
+    assert N * C * 4 >= 48 << 20  # where an eager call takes the second stream
+    sc = scenes.room_scene(n=N, C=C, seed=4)
+    cam = scenes.circle_poses(1, 320, 240, 262.5)[0]
+    ins = [dev(x) for x in (sc.means, sc.scales, sc.quats, sc.opacities, sc.rgb, sc.feats)]
+    fr = Frame([cam], sc.n, make_params(C=C, K=K), pair_capacity=1 << 21)
+    fr.bin_and_sort(*ins[:4])
+    F, rgb, T, ids = fr.new_outputs()
+    fr.render_forward(ins[4], ins[5], F, rgb, T, ids)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    dF, drgb = torch.randn(F.shape, generator=g, device="cuda"), torch.randn(rgb.shape, generator=g, device="cuda")
+    grads = [torch.empty_like(x) for x in ins]
+
+    def back():
+        fr.render_backward(*ins, T, dF, drgb, None, *grads)
+
+    back()
+    eager = []
+    for _ in range(3):
+        for x in grads:
+            x.fill_(7.0)
+        back()
+        eager.append([x.clone() for x in grads])  # read behind the call, on its stream
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        back()
+    for x in grads:
+        x.fill_(7.0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert fr.read_status()[0] == 0
+    for run in eager:
+        for a, b in zip(run, grads):
+            scale = b.abs().max().item()
+            assert scale > 0 and (a - b).abs().max().item() <= 1e-5 * scale
