@@ -607,14 +607,18 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
         // chunk b0 is worked on while the one before it is copied and the list entries of the next are read
         int b0 = ((L - 1) >> 5) << 5;  // (L = 0: the loop does not run)
         ListEntry e1 = list_entry(list, masks, b0 + lane, L);
-        uint32_t word = stage((b0 >> 5) & 1, e1), lower = 0u, lower_next = 0u;  // (H = 2: whose lower block is met)
-        if (H == 2) lower = __ballot_sync(ALL, (e1.mask & (1u << WX << wb)) != 0u);
+        uint32_t word = stage((b0 >> 5) & 1, e1), met[H] = {}, met_next[H] = {};  // (H = 2: those that each block meets)
+        auto blocks = [&](uint32_t (&m)[H]) {
+#pragma unroll
+            for (int i = 0; i < H; ++i) m[i] = __ballot_sync(ALL, (e1.mask & (1u << WX * i << wb)) != 0u);
+        };
+        if (H == 2) blocks(met);
         e1 = list_entry(list, masks, b0 - 32 + lane, L);
         for (; b0 >= 0 && L > 0; b0 -= 32) {
             const int buf = (b0 >> 5) & 1;
             const WarpStage& S = G.st[buf];
             const uint32_t next = stage(buf ^ 1, e1);
-            if (H == 2) lower_next = __ballot_sync(ALL, (e1.mask & (1u << WX << wb)) != 0u);
+            if (H == 2) blocks(met_next);
             e1 = list_entry(list, masks, b0 - 64 + lane, L);
             cp_async_wait_prev();  // this chunk's copies
             __syncwarp();
@@ -631,7 +635,7 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
                     sel[i] = false;
                     wsel[i] = 0.0f;
                     Hit h;
-                    if (H == 2 && i == 1 && !((lower >> j) & 1u)) continue;
+                    if (H == 2 && !((met[i] >> j) & 1u)) continue;  // as the forward, block by block
                     if (pos < nstop[i] &&
                         eval_splat<VAR>(S.r0[j], S.r1[j], S.r2[j], oc.x, pxf, pyf + (float)(4 * i), P.alpha_min, cam.near_plane, h,
                                         P.lowpass)) {
@@ -723,7 +727,8 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
                 }
             }
             word = next;
-            lower = lower_next;
+#pragma unroll
+            for (int i = 0; i < H; ++i) met[i] = met_next[i];
             __syncwarp();  // every lane has read this half before the next copies into it
         }
         cp_async_wait_all();

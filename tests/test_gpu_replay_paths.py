@@ -1,6 +1,7 @@
 """The backward replays at the sizes where their dispatch takes them: products shared by
 a warp's lanes with tiles of 8 and 16, in both types, on an image with enough blocks an SM (ragged to the
-right and below); and the feature rows written in the second stream after the replay.
+right and below); the feature rows written in the second stream after the replay; and a
+warp's two blocks, each with the surfels of its own warp mask.
 Gradients against the oracle's FP64 analytic ones, tolerances as in test_gpu_feat_grad_shapes.py;
 the second stream against the same call captured on one stream, tolerance as in
 test_gpu_autograd_graph.py (BF16 storage is not used).
@@ -9,9 +10,12 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2604_10951_gb300 import _lib as L
 from paper_2604_10951_gb300 import scenes
 from paper_2604_10951_gb300.raster import Frame, make_params
-from tests.gpu_util import dev
+from tests._scenes import ident_cam, make_scene
+from tests.gpu_util import GpuRun, dev
+from tests.test_gpu_backward import _gpu_backward
 from tests.test_gpu_feat_grad_shapes import _check
 
 pytestmark = pytest.mark.gpu
@@ -66,3 +70,28 @@ def test_feature_rows_in_the_second_stream_after_the_replay(N, C, K):
         for a, b in zip(run, grads):
             scale = b.abs().max().item()
             assert scale > 0 and (a - b).abs().max().item() <= 1e-5 * scale
+
+
+def test_a_block_without_its_mask_bit_is_not_replayed():
+    """Two blocks per warp: a surfel kept out of the upper block by the warp mask, as the
+    forward leaves it out there, gets nothing from that block's pixels in the replay either."""
+    W, H, K = 605, 413, 12
+    means = np.array([[0.0, 0.0, 2.0], [0.0, 0.0, 3.0]])
+    sc = make_scene(means, np.full((2, 2), 30.0), np.tile([1.0, 0.0, 0.0, 0.0], (2, 1)), np.array([0.5, 0.5]), C=8)
+    run = GpuRun(sc, [ident_cam(W=W, H=H, f=500.0)], K=K, render=False)
+    assert run.frame.region(L.REG_RANGES).numel() // 8 * 8 >= 48 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert run.ranges()[0].tolist() == [0, 2] and run.lists()[0] == 0
+    masks = run.frame.region(L.REG_MASK).view(torch.int32)
+    assert masks[0].item() == 0xff and masks[1].item() == 0xff
+    masks[0] = 0xfe  # tile (0, 0), block 0: without the nearer surfel
+    run.F, run.rgb_out, run.T, run.ids = run.frame.new_outputs()
+    run.frame.render_forward(run.rgb, run.feats, run.F, run.rgb_out, run.T, run.ids)
+    ids = run.view(0)["ids"]
+    assert ids[0, 0].tolist() == [1] + [-1] * (K - 1) and ids[4, 0].tolist() == [0, 1] + [-1] * (K - 2)
+    gT = np.zeros((H, W))
+    gT[0, 0] = 1.0
+    g = _gpu_backward(run, np.zeros((H, W, 8)), np.zeros((H, W, 3)), gT)
+    assert g["opac"][1] != 0.0 and g["opac"][0] == 0.0
+    gT[4, 0] = 1.0
+    g = _gpu_backward(run, np.zeros((H, W, 8)), np.zeros((H, W, 3)), gT)
+    assert g["opac"][0] != 0.0
