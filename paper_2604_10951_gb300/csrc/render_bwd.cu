@@ -740,8 +740,7 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
 // k_bwd_geo_full: the same replay for the full accumulation (K = 0)
 // ---------------------------------------------------------------------------
 // (TOPK: only the selected contributors, with the forward's weights; a surfel that none
-// of the warp's pixels selected costs no products, and a dL/dF that is not finite makes the
-// block leave out the products of pixels that did not select the surfel.)
+// of the warp's pixels selected costs no products.)
 // Every contributor takes the dot c_j . dL/dF and gives w dL/dF to its row.  The
 // block's dL/dF stays in registers for the whole walk, as PX pixels x 4 NQ channels
 // per lane (FullLanes: 8 x 8 at 64 channels), and serves both products: a lane's
@@ -749,7 +748,9 @@ __global__ void __launch_bounds__(geo_threads<TS, CF, FT, H>(),
 // them, which leaves each lane its own pixel's dot (7 shuffles for 8 pixels); with the
 // block's weights from shared memory a lane's channel sums are reduce-scattered over the
 // pixel groups and added to the surfel's row in L2 (256 consecutive bytes a warp at 64
-// channels).  The next surfel's row is read ahead.  640 x 480, 500k surfels, 64 channels
+// channels).  The next surfel's row is read ahead.  A dL/dF that is not finite would reach
+// the surfels that only other pixels of its block met, as -0 times it: such a block leaves
+// those products out.  640 x 480, 500k surfels, 64 channels
 // FP32: 481 us with a CTA per tile, all channels of a pixel in its lane and 95
 // shuffles per surfel for the sums, 246 here; the step with 16 channels 421 -> 339, 128
 // channels (spilled there) 2609 -> 811.  Bound by instruction issue.
@@ -844,17 +845,14 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                 df[p][q][1] = make_float2(f[q].z, f[q].w);
             }
         }
-        bool careful = false;  // TOPK: some dL/dF is not finite
-        if constexpr (TOPK) {
-            float2 z = make_float2(0.0f, 0.0f);
+        float2 z = make_float2(0.0f, 0.0f);  // NaN when some dL/dF is not finite
 #pragma unroll
-            for (int p = 0; p < PX; ++p)
+        for (int p = 0; p < PX; ++p)
 #pragma unroll
-                for (int q = 0; q < NQ; ++q)
+            for (int q = 0; q < NQ; ++q)
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) z = __ffma2_rn(df[p][q][k], make_float2(0.0f, 0.0f), z);
-            careful = __any_sync(ALL, !(z.x + z.y == 0.0f));
-        }
+                for (int k = 0; k < 2; ++k) z = __ffma2_rn(df[p][q][k], make_float2(0.0f, 0.0f), z);
+        const bool careful = __any_sync(ALL, !(z.x + z.y == 0.0f));
 
         // one chunk's records and gradient slots, and the lane mask of those the warp meets
         auto stage = [&](int buf, const ListEntry& e) {
@@ -987,7 +985,7 @@ __global__ void __launch_bounds__(full_threads<TS>(), (CMAX <= 64 ? 512 : 256) /
                                     sum[q][k] = __ffma2_rn(make_float2(wp[p], wp[p]), df[p][q][k], sum[q][k]);
                         }
                     };
-                    if (TOPK && careful) pixels(std::true_type{});
+                    if (careful) pixels(std::true_type{});
                     else pixels(std::false_type{});
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {

@@ -1,7 +1,7 @@
 """The backward replays at the sizes where their dispatch takes them: products shared by
 a warp's lanes with tiles of 8 and 16, in both types, on an image with enough blocks an SM (ragged to the
-right and below); the feature rows written in the second stream after the replay; and a
-warp's two blocks, each with the surfels of its own warp mask.
+right and below); the feature rows written in the second stream after the replay; a
+warp's two blocks, each with the surfels of its own warp mask; and a dL/dF that is not finite.
 Gradients against the oracle's FP64 analytic ones, tolerances as in test_gpu_feat_grad_shapes.py;
 the second stream against the same call captured on one stream, tolerance as in
 test_gpu_autograd_graph.py (BF16 storage is not used).
@@ -95,3 +95,19 @@ def test_a_block_without_its_mask_bit_is_not_replayed():
     gT[4, 0] = 1.0
     g = _gpu_backward(run, np.zeros((H, W, 8)), np.zeros((H, W, 3)), gT)
     assert g["opac"][0] != 0.0
+
+
+@pytest.mark.parametrize("C,ts", [(16, 16), (64, 16), (64, 8), (128, 32)])
+def test_an_infinite_gradient_without_a_selection(C, ts):
+    """Full accumulation: a pixel with an infinite dL/dF reaches the surfels that it met and no others."""
+    sc, cam = scenes.tiny_scene(seed=5, n=1200, C=C)
+    run = GpuRun(sc, [cam], K=0, tile_size=ts)
+    H, W = run.view(0)["T"].shape
+    zero = np.zeros((H, W, C))
+    y, x = np.argwhere(run.view(0)["T"] < 0.9)[0]
+    gF, one = zero.copy(), zero.copy()
+    gF[y, x] = np.inf
+    one[y, x] = 1.0
+    met = np.abs(_gpu_backward(run, one, zero[..., :3], zero[..., 0])["feat"]).max(-1) > 0
+    g = _gpu_backward(run, gF, zero[..., :3], zero[..., 0])
+    assert met.any() and np.array_equal(~np.isfinite(g["feat"]).all(-1), met)
