@@ -19,6 +19,15 @@ void kernel_mark(cudaStream_t s);
 // launch stream, one after another.
 bool kernel_marks_armed();
 
+// Opens a kernel to dynamic shared-memory requests above 48 KB: to all that it ever makes,
+// with room for its static shared memory (at most 7 KB) in the 227 KB of a CTA.  The limit
+// belongs to the kernel and not to a launch: set to each call's own request, a thread's smaller one took
+// effect between another thread's call and its launch, which was then refused.
+constexpr int SMEM_LIMIT = 220 * 1024;
+inline cudaError_t open_smem(const void* kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+}
+
 // A second stream of the calling thread on the current device, with a fork
 // and a join event, for work that may overlap the launch stream `s`.  False
 // when there is none (not created while `s` is being captured, or creation

@@ -264,7 +264,7 @@ cudaError_t launch_kc(int64_t N, int nq, const void* f_ins, const float* means, 
     auto kern = k_query_labels<KC>;
     cudaError_t e = cudaSuccess;
     if (smem + 1024 > 48 * 1024) {  // with the static shared memory
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = open_smem((const void*)kern);
         if (e != cudaSuccess) return e;
     }
     // resident CTAs per SM from the kernel's registers and shared memory (the

@@ -357,7 +357,7 @@ cudaError_t launch_qb(int64_t N, int nq, int dim, int ncols, int nbuf, const voi
     // another one has done all its tiles (865k x 144 x 32 in FP32: 306 us, 195.02 without)
     const int per_sm = std::max(1, std::min({QB == 2 ? 2 : 3, 512 / (QB * ncols), (int)(227 * 1024 / (smem + 4 * 1024))}));
     smem = std::max(smem, (size_t)(227 * 1024 / (per_sm + 1)));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = open_smem((const void*)kern);
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (N + QM * QB - 1) / (QM * QB);
     const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms);

@@ -1270,10 +1270,7 @@ __global__ void __launch_bounds__(256) k_bwd_clear(const __grid_constant__ Cams 
 // ---------------------------------------------------------------------------
 namespace {
 
-cudaError_t set_smem(const void* k, size_t smem) {
-    if (smem > 48 * 1024) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return cudaSuccess;
-}
+cudaError_t set_smem(const void* k, size_t smem) { return smem > 48 * 1024 ? open_smem(k) : cudaSuccess; }
 
 // one resident wave: CTAs per SM times SMs, capped by the number of tiles
 cudaError_t persistent_grid(const void* k, int threads, size_t smem, int& grid) {

@@ -505,7 +505,7 @@ inline cudaError_t launch_tiles(KernelT kern, int threads, size_t smem, const Ca
                                const AuxOut& x, int num_sms, cudaStream_t stream, int parts = 1) {
     cudaError_t e = cudaSuccess;
     if (smem + 2048 > 48 * 1024) {  // above the default limit with the kernels' static shared memory (< 2 KB)
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = open_smem((const void*)kern);
         if (e != cudaSuccess) return e;
     }
     int64_t units = (int64_t)cams.total_tiles * parts;
