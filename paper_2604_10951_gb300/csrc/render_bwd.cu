@@ -1270,7 +1270,8 @@ __global__ void __launch_bounds__(256) k_bwd_clear(const __grid_constant__ Cams 
 // ---------------------------------------------------------------------------
 namespace {
 
-cudaError_t set_smem(const void* k, size_t smem) { return smem > 48 * 1024 ? open_smem(k) : cudaSuccess; }
+// (the 48 KB that need no attribute include the kernel's static shared memory, under 1 KB)
+cudaError_t set_smem(const void* k, size_t smem) { return smem + 1024 > 48 * 1024 ? open_smem(k) : cudaSuccess; }
 
 // one resident wave: CTAs per SM times SMs, capped by the number of tiles
 cudaError_t persistent_grid(const void* k, int threads, size_t smem, int& grid) {

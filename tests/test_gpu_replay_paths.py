@@ -1,7 +1,8 @@
 """The backward replays at the sizes where their dispatch takes them: products shared by
 a warp's lanes with tiles of 8 and 16, in both types, on an image with enough blocks an SM (ragged to the
 right and below); the feature rows written in the second stream after the replay; a
-warp's two blocks, each with the surfels of its own warp mask; and a dL/dF that is not finite.
+warp's two blocks, each with the surfels of its own warp mask; a dL/dF that is not finite; and the
+feature kernel where its shared memory with the static part just exceeds 48 KB.
 Gradients against the oracle's FP64 analytic ones, tolerances as in test_gpu_feat_grad_shapes.py;
 the second stream against the same call captured on one stream, tolerance as in
 test_gpu_autograd_graph.py (BF16 storage is not used).
@@ -111,3 +112,9 @@ def test_an_infinite_gradient_without_a_selection(C, ts):
     met = np.abs(_gpu_backward(run, one, zero[..., :3], zero[..., 0])["feat"]).max(-1) > 0
     g = _gpu_backward(run, gF, zero[..., :3], zero[..., 0])
     assert met.any() and np.array_equal(~np.isfinite(g["feat"]).all(-1), met)
+
+
+@pytest.mark.parametrize("C,dtype,K,ts", [(12, torch.float32, 5, 16), (48, torch.float32, 4, 8)])
+def test_feature_kernel_just_above_48_kb(C, dtype, K, ts):
+    sc, cam = scenes.tiny_scene(seed=71 + C, n=600, C=C)
+    _check(sc, cam, K, dtype, tile_size=ts, seed=C)
