@@ -439,12 +439,12 @@ def device_scene(torch, dev, sc):
 # pose 0, the L2 contents the step's earlier kernels left; ncu --cache-control none),
 # from the in-step traffic summary under profiles/; to be set to None whenever the
 # kernel changes after that capture
-NCU_TRAFFIC = {"k_render_topk": 55170304 + 109097728, "k_bwd_feat": 19863296 + 24290304,
-               "k_bwd_geo": 13771264 + 9980928}
+NCU_TRAFFIC = {"k_render_topk": 55720960 + 104460544, "k_bwd_feat": 19561216 + 24040960,
+               "k_bwd_geo": 13892608 + 9878016}
 # (smsp__inst_executed.sum, gpu__time_duration.sum in us) of the one-kernel
 # captures summarised under profiles/
-NCU_ISSUE = {"k_render_topk": (81518618, 108.0), "k_bwd_feat": (61610201, 76.608),
-             "k_bwd_geo": (78331788, 89.056)}
+NCU_ISSUE = {"k_render_topk": (81518618, 105.28), "k_bwd_feat": (61610201, 76.352),
+             "k_bwd_geo": (78331788, 90.816)}
 # the query-label kernel's capture (summarised under profiles/): DRAM read + write
 NCU_QUERY_TRAFFIC = {"nq32_dim32_f32": 47276544}
 

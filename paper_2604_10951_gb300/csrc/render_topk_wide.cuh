@@ -21,7 +21,7 @@
 //     consecutive entries (a thread per pixel would write 4 K bytes apart).
 // 1296 x 968, K = 24, C = 16 FP32, 500k surfels: 1400 us with the set in
 // registers (8 warps per SM, 1.49 instructions per cycle), 558 us here (20
-// warps, 2.02); now bound by the shared-memory path (73 % busy: four 16-byte
+// warps, 2.04); now bound by the shared-memory path (76 % busy: four 16-byte
 // record reads per evaluation, the set, three reads per selected row chunk).
 #pragma once
 
