@@ -118,3 +118,18 @@ def test_an_infinite_gradient_without_a_selection(C, ts):
 def test_feature_kernel_just_above_48_kb(C, dtype, K, ts):
     sc, cam = scenes.tiny_scene(seed=71 + C, n=600, C=C)
     _check(sc, cam, K, dtype, tile_size=ts, seed=C)
+
+
+@pytest.mark.parametrize("C,dtype,ts", [(64, torch.float32, 8), (64, torch.bfloat16, 16), (128, torch.float32, 16)])
+def test_an_infinite_gradient_with_products_on_small_tiles(C, dtype, ts):
+    """Top-K: only the surfels that the pixel selected."""
+    W, H, K = 321, 243, 24
+    sc, cam = scenes.tiny_scene(seed=5, n=1200, C=C)
+    s = W / cam.width
+    run = GpuRun(sc, [scenes.Camera(cam.fx * s, cam.fy * s, W / 2, H / 2, W, H, cam.viewmat)], K=K, tile_size=ts, feat_dtype=dtype)
+    ids = run.view(0)["ids"]
+    gF = np.ones((H, W, C))
+    y, x = np.argwhere((ids >= 0).any(-1))[0]
+    gF[y, x] = np.inf
+    g = _gpu_backward(run, gF, np.zeros((H, W, 3)), np.zeros((H, W)), feat_dtype=dtype)
+    assert np.array_equal(np.flatnonzero(~np.isfinite(g["feat"]).all(-1)), np.unique(ids[y, x][ids[y, x] >= 0]))
